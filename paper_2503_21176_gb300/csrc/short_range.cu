@@ -8,9 +8,11 @@
 // k_theta, eps and s are the SPC/Fw values (Wu, Tepper & Voth, J. Chem. Phys.
 // 124, 024503 (2006)) converted from kcal/mol to eV.
 // Intramolecular terms: one thread per molecule (minimum image).  Lennard-Jones:
-// one thread per sorted O atom over its ELLPACK row (both directions of a pair
+// one warp per sorted O atom over its ELLPACK row (both directions of a pair
 // are visited, so the energy takes 1/2), with the current positions and the
 // images of the list.
+#include <algorithm>
+
 #include "internal.cuh"
 
 namespace qeq {
@@ -71,54 +73,112 @@ __global__ void k_water_intra(int n_mol, const double *__restrict__ R, double Lx
     if (threadIdx.x == 0) part[blockIdx.x] = vals[0];
 }
 
-// O-O Lennard-Jones over the list, one block per brick: sorted atom i is an O
-// when perm[i] % 3 == 0; an entry e of row i is decoded through the brick's tile
-// table into the sorted atom j and its image shift.
-__global__ void __launch_bounds__(kThreads)
-k_water_lj(int n, BrickGeom g, const int32_t *__restrict__ cell_start,
-           const int32_t *__restrict__ perm, const uint16_t *__restrict__ nbr,
-           const int32_t *__restrict__ cnt, const double *__restrict__ R,
-           const double *__restrict__ wrap_off, double Lx, double Ly, double Lz, double rc2,
-           double *__restrict__ F, double *__restrict__ part) {
-    __shared__ int t_start[kMaxTileBricks], t_base[kMaxTileBricks], t_code[kMaxTileBricks], t_total;
+// O-O Lennard-Jones over the list: nchunk blocks per brick, one warp per O row
+// (sorted atom i is an O when perm[i] % 3 == 0).  A lane takes 4 entries of a
+// stripe (one 8-byte word), 8 stripes a warp, decodes them through the brick's
+// tile table (written by the neighbour build) into the sorted atom j and its
+// image, and the warp packs its O neighbours (a third of the entries) into a
+// shared queue, 32 of which are then evaluated together.  GB300 runs FP64 at
+// 1/64 of FP32, so the pair term is bound by FP64 issue slots: packed, they run
+// on full warps.  One thread per row over its whole list, one block per brick,
+// waited on a chain of dependent loads per entry and left most of the chip idle:
+// 722 us of the 1,705 us FP64 step of 648 atoms (r_c 9 A), which takes 1,030 us now.
+constexpr int kLjThreads = 256;
+constexpr int kLjQueue = 160;  // up to 31 left over and 4 x 32 new entries
+
+__global__ void __launch_bounds__(kLjThreads)
+k_water_lj(int n, BrickGeom g, int nchunk, const int4 *__restrict__ tile_tab,
+           const int32_t *__restrict__ cell_start, const int32_t *__restrict__ perm,
+           const uint16_t *__restrict__ nbr, const int32_t *__restrict__ cnt,
+           const double *__restrict__ R, const double *__restrict__ wrap_off, double Lx, double Ly,
+           double Lz, double rc2, double *__restrict__ F, double *__restrict__ part) {
+    __shared__ int t_start[kMaxTileBricks], t_base[kMaxTileBricks], t_code[kMaxTileBricks];
+    __shared__ int queue[kLjThreads / 32][kLjQueue];  // atom j | image code << 24
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    constexpr int nw = kLjThreads / 32;
+    int *qu = queue[warp];
     double e = 0.0;
     const double s6 = kLjSigma * kLjSigma * kLjSigma * kLjSigma * kLjSigma * kLjSigma;
-    for (int64_t b = blockIdx.x; b < g.nbricks; b += gridDim.x) {
+    const int64_t units = g.nbricks * nchunk;
+    for (int64_t w = blockIdx.x; w < units; w += gridDim.x) {
+        const int64_t b = w / nchunk;
+        const int chunk = (int)(w - b * nchunk);
         __syncthreads();
-        if (threadIdx.x < 32) tile_table(g, b, cell_start, t_start, t_base, t_code, &t_total);
+        for (int rb = threadIdx.x; rb < g.T; rb += kLjThreads) {
+            const int4 t = tile_tab[b * g.T + rb];
+            t_start[rb] = t.x;
+            t_base[rb] = t.y;
+            t_code[rb] = t.z;
+        }
         __syncthreads();
-        const int i0 = t_start[g.center], i1 = cell_start[(b + 1) * g.bvol];
-        for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
+        const int i0 = cell_start[b * g.bvol], i1 = cell_start[(b + 1) * g.bvol];
+        for (int i = i0 + chunk * nw + warp; i < i1; i += nchunk * nw) {
             const int ai = perm[i];
             if (ai % 3 != 0) continue;
             const double xi = R[3 * (size_t)ai] + wrap_off[3 * (size_t)ai];
             const double yi = R[3 * (size_t)ai + 1] + wrap_off[3 * (size_t)ai + 1];
             const double zi = R[3 * (size_t)ai + 2] + wrap_off[3 * (size_t)ai + 2];
             double fx = 0.0, fy = 0.0, fz = 0.0;
-            const int c = cnt[i];
-            for (int k = 0; k < c; ++k) {
-                const int en = nbr[list_index(k, i, n)];
-                const int rb = tile_locate(en, g.T, t_start, t_base);
-                const int aj = perm[en - t_base[rb]];
-                if (aj % 3 != 0) continue;
-                const int code = t_code[rb];
+            auto pair = [&](int v) {
+                const int aj = v & kIndexMask, code = v >> kIndexBits;
                 const double dx = (R[3 * (size_t)aj] + wrap_off[3 * (size_t)aj] - xi) + (code / 25 - 2) * Lx;
                 const double dy = (R[3 * (size_t)aj + 1] + wrap_off[3 * (size_t)aj + 1] - yi) +
                                   ((code / 5) % 5 - 2) * Ly;
                 const double dz = (R[3 * (size_t)aj + 2] + wrap_off[3 * (size_t)aj + 2] - zi) +
                                   (code % 5 - 2) * Lz;
                 const double r2 = dx * dx + dy * dy + dz * dz;
-                if (!(r2 < rc2)) continue;
-                const double inv6 = s6 / (r2 * r2 * r2);
+                if (!(r2 < rc2)) return;
+                const double ir2 = 1.0 / r2;
+                const double inv6 = s6 * (ir2 * ir2 * ir2);
                 e += 0.5 * 4.0 * kLjEps * (inv6 * inv6 - inv6);
-                const double gg = 4.0 * kLjEps * (-12.0 * inv6 * inv6 + 6.0 * inv6) / r2;
+                const double gg = 4.0 * kLjEps * (-12.0 * inv6 * inv6 + 6.0 * inv6) * ir2;
                 fx += gg * dx;
                 fy += gg * dy;
                 fz += gg * dz;
+            };
+            const int c = cnt[i];
+            const int sub = lane % kListLanes;
+            int nq = 0;
+            for (int k0 = (lane / kListLanes) * kListStripe; __any_sync(0xffffffffu, k0 < c);
+                 k0 += 32 / kListLanes * kListStripe) {
+                // this lane's entries k0 + sub + 4 u of the stripe that starts at k0
+                uint2 wd = make_uint2(0u, 0u);
+                if (k0 + sub < c) wd = *(const uint2 *)(nbr + list_index(k0 + sub, i, n));
+                const int ev[4] = {(int)(wd.x & 0xffffu), (int)(wd.x >> 16), (int)(wd.y & 0xffffu),
+                                   (int)(wd.y >> 16)};
+                int found[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    found[u] = -1;
+                    if (k0 + sub + kListLanes * u < c) {
+                        const int rb = tile_locate(ev[u], g.T, t_start, t_base);
+                        const int aj = perm[ev[u] - t_base[rb]];
+                        if (aj % 3 == 0) found[u] = aj | (t_code[rb] << kIndexBits);
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const unsigned m = __ballot_sync(0xffffffffu, found[u] >= 0);
+                    if (found[u] >= 0) qu[nq + __popc(m & ((1u << lane) - 1u))] = found[u];
+                    nq += __popc(m);
+                }
+                __syncwarp();
+                while (nq >= 32) {
+                    nq -= 32;
+                    pair(qu[nq + lane]);
+                }
+                __syncwarp();
             }
-            F[3 * (size_t)ai] += fx;
-            F[3 * (size_t)ai + 1] += fy;
-            F[3 * (size_t)ai + 2] += fz;
+            if (lane < nq) pair(qu[lane]);
+            __syncwarp();
+            fx = warp_sum(fx);
+            fy = warp_sum(fy);
+            fz = warp_sum(fz);
+            if (lane == 0) {
+                F[3 * (size_t)ai] += fx;
+                F[3 * (size_t)ai + 1] += fy;
+                F[3 * (size_t)ai + 2] += fz;
+            }
         }
     }
     double vals[1] = {e};
@@ -136,9 +196,15 @@ int short_range_forces(qeq_ctx *ctx, const double *R, const double *, double *F_
     const qeq_params &p = ctx->p;
     k_water_intra<<<ctx->red_grid, kThreads, 0, s>>>(n / 3, R, p.box[0], p.box[1], p.box[2], F_short,
                                                   ctx->part);
-    k_water_lj<<<ctx->red_grid, kThreads, 0, s>>>(n, ctx->geom, ctx->cell_start, ctx->perm, ctx->nbr,
-                                               ctx->cnt, R, ctx->wrap_off, p.box[0], p.box[1],
-                                               p.box[2], p.r_cut * p.r_cut, F_short, ctx->part);
+    // blocks per brick: as many as fill the grid when the box has few bricks, at
+    // most one per 8 rows (a warp a row)
+    const int64_t nb = ctx->geom.nbricks;
+    const int nchunk = (int)std::max<int64_t>(
+        1, std::min<int64_t>(ctx->red_grid / nb, (ctx->max_rows + kLjThreads / 32 - 1) / (kLjThreads / 32)));
+    k_water_lj<<<ctx->red_grid, kLjThreads, 0, s>>>(n, ctx->geom, nchunk, ctx->tile_tab, ctx->cell_start,
+                                                    ctx->perm, ctx->nbr, ctx->cnt, R, ctx->wrap_off,
+                                                    p.box[0], p.box[1], p.box[2], p.r_cut * p.r_cut,
+                                                    F_short, ctx->part);
     launch_finalize(ctx, ctx->part, 2, e_slot, s);
     ctx->launches += 3;
     return cuda_check(ctx, cudaGetLastError(), "short-range launch");
