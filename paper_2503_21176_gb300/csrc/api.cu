@@ -168,6 +168,7 @@ int create(const qeq_params *p, cudaStream_t stream, bool async_alloc, qeq_ctx *
         ctx->sm_count = sms;
         ctx->red_grid = std::min(kRedBlocks, kRedPerSm * sms);
     }
+    ctx->atom_grid = std::min(ctx->red_grid, grid_for(ctx->n));
     cudaGetLastError();
     rc = nl_configure(ctx);
     if (!rc) rc = nl_alloc(ctx);

@@ -541,7 +541,7 @@ int shadow_evaluate(qeq_ctx *ctx, const qeq_md_params *prm, qeq_md_state *st, cu
     double *nn = st->n_hist;  // n(t) is history slot 0
     double *part = ctx->part;
     double *scal = ctx->scal;
-    const int G = ctx->red_grid;
+    const int G = ctx->atom_grid;
     unsigned int *tk = ctx->ticket;
     auto fin = [&]() { ctx->launches += 1; };  // a reducing kernel (its last block finalizes)
 
@@ -586,7 +586,7 @@ int shadow_evaluate(qeq_ctx *ctx, const qeq_md_params *prm, qeq_md_state *st, cu
     auto solve_rank = [&](int k, bool *done) -> int {
         const int nO = k * (k + 1) / 2;
         prof_begin(ctx, kPhShadow, s);
-        launch_normal_part(ctx->pdl, ctx->red_grid, k, n, ctx->Rb, ctx->fvec, part, ctx->p.q_tot, k + 1, scal,
+        launch_normal_part(ctx->pdl, G, k, n, ctx->Rb, ctx->fvec, part, ctx->p.q_tot, k + 1, scal,
                            st->energies, tk, s);
         ctx->launches += 1;
         prof_end(ctx, s);
@@ -658,7 +658,7 @@ int shadow_evaluate(qeq_ctx *ctx, const qeq_md_params *prm, qeq_md_state *st, cu
 int shadow_advance_queue(qeq_ctx *ctx, const qeq_md_params *prm, qeq_md_state *st, cudaStream_t s) {
     const int n = (int)ctx->n;
     prof_begin(ctx, kPhIntegrate, s);
-    launch_pdl(ctx->pdl, k_advance, ctx->red_grid, kThreads, 0, s, n, ctx->p.dt, 0.5 * ctx->p.dt,
+    launch_pdl(ctx->pdl, k_advance, ctx->atom_grid, kThreads, 0, s, n, ctx->p.dt, 0.5 * ctx->p.dt,
                ctx->p.mass_unit, dissipation(ctx->p.dissipation_k), prm->mass, st->F, st->Kf, st->R,
                st->V, st->n_hist, ctx->half_kick, ctx->R_build, ctx->part, ctx->scal + kScMaxDisp2,
                ctx->ticket);
@@ -688,7 +688,7 @@ int shadow_finish(qeq_ctx *ctx, const qeq_md_params *prm, qeq_md_state *st, bool
     const int n = (int)ctx->n;
     prof_begin(ctx, kPhIntegrate, s);
     const int rank = kf && st->Kf ? ctx->kf_rank : 0;
-    launch_pdl(ctx->pdl, k_finish, ctx->red_grid, kThreads, 0, s, n, 0.5 * ctx->p.mass_unit, kick, prm->mass,
+    launch_pdl(ctx->pdl, k_finish, ctx->atom_grid, kThreads, 0, s, n, 0.5 * ctx->p.mass_unit, kick, prm->mass,
                ctx->half_kick, st->F, st->V, rank, ctx->Wb, st->Kf, ctx->part, ctx->scal,
                st->energies, ctx->ticket);
     prof_end(ctx, s);

@@ -17,7 +17,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("n_mol,r_cut,skin", [(1, 1.2, 0.2), (9, 4.0, 0.5), (64, 9.0, 1.0), (216, 9.0, 1.0),
-                                              (1001, 6.0, 0.5), (4000, 5.0, 0.3)])
+                                              (1001, 6.0, 0.5), (1728, 5.0, 0.3)])
 def test_water_term_matches_oracle(n_mol, r_cut, skin):
     qg = cuda_or_skip()
     w = water_box(n_mol, seed=100 + n_mol)
