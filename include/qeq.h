@@ -530,7 +530,18 @@ int qeq_pair_table_eval(double alpha, double smax, int32_t which, int64_t n, con
                         double *F, double *G, int32_t *in_table, int32_t *kept);
 
 /*
- * Diagnostic: the same evaluation on the device, with the tables of an FP64
+ * Diagnostic, host only: pairs as the FP64 real-space kernel evaluates them in
+ * fixed point, for n displacements d [n][3] with widths sigma_i, sigma_j [n] (host
+ * arrays; |d| below twice the cutoff).  path[k] = 1: f[k] = erfc(alpha r) / r - erfc(r / gamma) / r and gc[k] =
+ * (df/dr) / r; 0: a pair the kernel leaves to its exact FP64 path (f, gc untouched);
+ * -1: beyond the cutoff.  QEQ_ERR_INVALID for a bad argument.
+ */
+int qeq_fixed_pair_eval(double alpha, double r_cut, int64_t n, const double *d,
+                        const double *sigma_i, const double *sigma_j, double *f, double *gc,
+                        int32_t *path);
+
+/*
+ * Diagnostic: qeq_pair_table_eval on the device, with the tables of an FP64
  * context (which as in qeq_pair_table_eval); arg, F, G, in_table are device
  * arrays of n entries.  QEQ_ERR_INVALID for an FP32-mixed context.
  */

@@ -156,6 +156,8 @@ def load(build_if_missing: bool = True) -> ctypes.CDLL:
     L.qeq_pair_table_eval.argtypes = [ctypes.c_double, ctypes.c_double, ctypes.c_int32, ctypes.c_int64,
                                       P, P, P, P, ctypes.POINTER(ctypes.c_int32)]
     L.qeq_pair_table_eval.restype = ctypes.c_int
+    L.qeq_fixed_pair_eval.argtypes = [ctypes.c_double, ctypes.c_double, ctypes.c_int64, P, P, P, P, P, P]
+    L.qeq_fixed_pair_eval.restype = ctypes.c_int
     L.qeq_selftest_pair64.argtypes = [P, ctypes.c_int32, P, P, P, P, ctypes.c_int64, P]
     L.qeq_selftest_pair64.restype = ctypes.c_int
     SI = ctypes.POINTER(qeq_solve_info)
@@ -474,6 +476,22 @@ def qeq_pair_table_eval(alpha, smax, which, arg):
     _check(None, load().qeq_pair_table_eval(float(alpha), float(smax), int(which), a.size, ptr(a),
                                             ptr(F), ptr(G), ptr(inn), ctypes.byref(kept)))
     return F, G, inn, int(kept.value)
+
+
+def qeq_fixed_pair_eval(alpha, r_cut, d, sigma_i, sigma_j):
+    """Pairs as the FP64 real-space kernel evaluates them in fixed point (host only).
+
+    d: [n, 3] displacements.  Returns (f, gc, path); f, gc are NaN where path is not 1."""
+    import numpy as np
+
+    d = np.ascontiguousarray(d, dtype=np.float64)
+    si, sj = (np.ascontiguousarray(np.broadcast_to(s, len(d)), dtype=np.float64) for s in (sigma_i, sigma_j))
+    f, gc = np.full(len(d), np.nan), np.full(len(d), np.nan)
+    path = np.zeros(len(d), dtype=np.int32)
+    ptr = lambda x: ctypes.c_void_p(x.ctypes.data)
+    _check(None, load().qeq_fixed_pair_eval(float(alpha), float(r_cut), len(d), ptr(d), ptr(si), ptr(sj),
+                                            ptr(f), ptr(gc), ptr(path)))
+    return f, gc, path
 
 
 def qeq_selftest_pair64(ctx, which, arg, F, G, in_table, stream=None) -> None:

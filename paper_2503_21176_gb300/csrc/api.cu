@@ -603,6 +603,21 @@ QEQ_API int qeq_pair_table_eval(double alpha, double smax, int32_t which, int64_
     return pair_table_eval_host(which, alpha, smax, n, arg, F, G, in_table, kept);
 }
 
+namespace qeq {
+int fixed_pair_eval_host(double alpha, double r_cut, int64_t n, const double *d, const double *si,
+                         const double *sj, double *f, double *gc, int32_t *path);
+}
+
+QEQ_API int qeq_fixed_pair_eval(double alpha, double r_cut, int64_t n, const double *d,
+                                const double *sigma_i, const double *sigma_j, double *f, double *gc,
+                                int32_t *path) {
+    if (n < 0 || (n > 0 && (!d || !sigma_i || !sigma_j || !f || !gc || !path)))
+        return set_error(nullptr, QEQ_ERR_INVALID, "fixed_pair_eval: bad argument");
+    if (!(alpha > 0.0 && r_cut > 0.0) || !std::isfinite(alpha) || !std::isfinite(r_cut))
+        return set_error(nullptr, QEQ_ERR_INVALID, "fixed_pair_eval: alpha and r_cut must be positive");
+    return fixed_pair_eval_host(alpha, r_cut, n, d, sigma_i, sigma_j, f, gc, path);
+}
+
 QEQ_API int qeq_selftest_pair64(qeq_ctx *ctx, int32_t which, const double *arg, double *F, double *G,
                                 int32_t *in_table, int64_t n, void *stream) {
     if (!ctx) return QEQ_ERR_INVALID;

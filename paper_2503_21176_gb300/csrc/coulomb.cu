@@ -4,7 +4,7 @@
 // Gaussian-charge correction) + smooth PME (Alg. 2) + self term (Eq. ewald_self).
 // Launch sequence per apply, all on the caller's stream:
 //   gather_in   sorted copies (x, y, z, q), sigma and B-spline base/fraction
-//   real        one thread per sorted atom over its ELLPACK row (no atomics)
+//   real        four or more lanes per sorted atom over its ELLPACK row (no atomics)
 //   spread      one thread per sorted atom, p^3 atomic adds onto the K^3 mesh
 //   cuFFT R2C   (library call)
 //   influence   Q^ *= G on the half spectrum, plus the mesh energy partial sums
@@ -13,23 +13,42 @@
 //               the real-space part and written in original atom order, with
 //               energy partial sums
 //   finalize    one block per energy component (fixed-order, deterministic)
-// FP64 mode runs all of it in double.  FP32_MIXED runs the pair math, the
+// FP64 mode runs all of it in double, the pair sum in 64-bit fixed point of FP64's
+// accuracy (real64_fixed.cuh).  FP32_MIXED runs the pair math, the
 // spreading, the FFT and the gather in float.  It accumulates rows in float
 // chunks of 32 flushed into double, and keeps the energies and outputs in double.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <tuple>
 #include <map>
+#include <memory>
 #include <mutex>
 #include <new>
 #include <type_traits>
 #include <vector>
 
+#include "fixed64.cuh"
+#include "fixed64_tables.h"
 #include "internal.cuh"
 
 namespace qeq {
 
 namespace {
+
+// What the FP64 gathers write for the fixed-point real space (x null: nothing).
+struct FxGather {
+    ulonglong4_32a *x;
+    u64 *s2;
+    int coord_bits, sigma_bits;
+};
+
+// Raises the flag to the largest biased exponent of the warp's charges (all lanes
+// call; q = 0 outside the atoms).
+__device__ __forceinline__ void fx_charge_exponent(double q, int32_t *flags) {
+    const int ex = __reduce_max_sync(0xffffffffu, (__double2hiint(q) >> 20) & 0x7FF);
+    if ((threadIdx.x & 31) == 0 && ex > 0) atomicMax(&flags[kFlagChargeExp], ex);
+}
 
 template <typename T> struct V4;
 template <> struct V4<double> { using type = double4_32a; };
@@ -80,10 +99,19 @@ __global__ void k_gather_in(int n, const int32_t *__restrict__ perm, const doubl
                             const double *__restrict__ sigma, double sK0, double sK1, double sK2,
                             typename V4<T>::type *__restrict__ xq, T *__restrict__ sg,
                             int4 *__restrict__ sbase, typename V4<T>::type *__restrict__ sfrac,
-                            int32_t *__restrict__ smax_bits, float4 *__restrict__ xf,
+                            int32_t *__restrict__ smax_bits, float4 *__restrict__ xf, FxGather fx,
                             int32_t *__restrict__ flags) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (smax_bits) {
+    if constexpr (std::is_same<T, double>::value) {
+        if (fx.x) {
+            const bool in = i < n && QEQ_IN_BOUNDS((unsigned)perm[i] < (unsigned)n, flags, kSiteGatherPerm);
+            fx_charge_exponent(in ? q[perm[i]] : 0.0, flags);
+            const u64 s2 = in ? fx_sigma2(sigma[perm[i]], fx.sigma_bits) : 0ull;
+            if (in) fx.s2[i] = s2;
+            const int b = __reduce_max_sync(0xffffffffu, (int)fx_hi(s2));
+            if ((threadIdx.x & 31) == 0 && b > 0) atomicMax(smax_bits, b);
+        }
+    } else if (smax_bits) {
         // max |sigma| as float bits (non-negative floats order like their bits)
         int32_t b = i < n && QEQ_IN_BOUNDS((unsigned)perm[i] < (unsigned)n, flags, kSiteGatherPerm)
                         ? __float_as_int(f64_to_f32_trunc(sigma[perm[i]])) & 0x7FFFFFFF
@@ -117,6 +145,14 @@ __global__ void k_gather_in(int n, const int32_t *__restrict__ perm, const doubl
     } else {
         xq[i] = {(T)x, (T)y, (T)z, (T)qa};
         if (xf) xf[i] = make_float4((float)x, (float)y, (float)z, 0.0f);
+        if (fx.x) {
+            ulonglong4_32a f;
+            f.x = fx_from_double(x, fx.coord_bits);
+            f.y = fx_from_double(y, fx.coord_bits);
+            f.z = fx_from_double(z, fx.coord_bits);
+            f.w = (u64)__double_as_longlong(qa);
+            fx.x[i] = f;
+        }
         sg[i] = (T)sigma[a];
         const double fx = floor(ux), fy = floor(uy), fz = floor(uz);
         sbase[i] = make_int4((int)fx, (int)fy, (int)fz, 0);
@@ -129,15 +165,21 @@ __global__ void k_gather_in(int n, const int32_t *__restrict__ perm, const doubl
 template <typename T>
 __global__ void k_gather_q(int n, const int32_t *__restrict__ perm, const double *__restrict__ q,
                            typename V4<T>::type *__restrict__ xq,
-                           typename V4<T>::type *__restrict__ sfrac, int32_t *__restrict__ flags) {
+                           typename V4<T>::type *__restrict__ sfrac, FxGather fx,
+                           int32_t *__restrict__ flags) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    if (!QEQ_IN_BOUNDS((unsigned)perm[i] < (unsigned)n, flags, kSiteGatherPerm)) return;
-    T qa;
-    if constexpr (std::is_same<T, float>::value)
-        qa = f64_to_f32_trunc(q[perm[i]]);  // as k_gather_in, on the integer pipe
-    else
-        qa = q[perm[i]];
+    const bool in = i < n && QEQ_IN_BOUNDS((unsigned)perm[i] < (unsigned)n, flags, kSiteGatherPerm);
+    T qa = T(0);
+    if constexpr (std::is_same<T, float>::value) {
+        if (in) qa = f64_to_f32_trunc(q[perm[i]]);  // as k_gather_in, on the integer pipe
+    } else {
+        if (in) qa = q[perm[i]];
+        if (fx.x) {
+            fx_charge_exponent(qa, flags);
+            if (in) fx.x[i].w = (u64)__double_as_longlong(qa);
+        }
+    }
+    if (!in) return;
     xq[i].w = qa;
     sfrac[i].w = qa;
 }
@@ -381,7 +423,9 @@ __device__ __forceinline__ void gauss_corr64(double r2, double si2, double sj,
 // kErfcXMax^2 with the margin of the FP32 Gaussian-correction test.
 constexpr float kGaussTest = (float)(kErfcXMax * kErfcXMax * (1.0 + 1e-5));
 
-// FP64 real space, one block per brick, kTPR lanes per row.  Dynamic shared
+// FP64 real space on the FP64 pipe, where k_real64_fixed does not apply (a skin
+// beyond about the cutoff, a tile beyond 3,000 atoms).  One block per brick, kTPR
+// lanes per row.  Dynamic shared
 // memory holds the two pair-function tables, the tile (double4 positions with
 // q, double sigma, float4 positions for the FP32 prefilter; GTILE: in the
 // block's slice of a global scratch buffer instead) and the per-lane queues of
@@ -540,6 +584,8 @@ k_real64(RealArgs a, BrickGeom g, const int4 *__restrict__ tile_tab, const int32
         }
     }
 }
+
+#include "real64_fixed.cuh"
 
 // Self-test hook: the FP64 piecewise erfc and its derivative on n device inputs.
 __global__ void k_erfc64(int64_t n, const double *__restrict__ tab, const double *__restrict__ x,
@@ -1074,6 +1120,7 @@ struct GatherArgs {
     double self_coef;   // k_e * (-2 alpha / sqrt(pi))
     double gauss_coef;  // k_e * sqrt(2 / pi) when the Gaussian self-energy is on, else 0
     float sx_f, sy_f, sz_f, self_coef_f, gauss_coef_f;  // FP32 copies (FP32-mixed epilogue)
+    int32_t *charge_exp;  // cleared for the next apply (after this one's real space), or null
 };
 
 
@@ -1093,6 +1140,7 @@ k_gather_out(GatherArgs a, const int32_t *__restrict__ perm, const int4 *__restr
              double *__restrict__ F_out, double *__restrict__ part) {
     // FP32-mixed: the real-space kernel left (v, E) as one float4 per sorted atom
     const float4 *vE32 = reinterpret_cast<const float4 *>(E_s);
+    if (a.charge_exp && blockIdx.x == 0 && threadIdx.x == 0) *a.charge_exp = 0;
     double e_tot = 0.0, e_real = 0.0, e_self = 0.0;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < a.n; i += gridDim.x * blockDim.x) {
         const int4 b = sbase[i];
@@ -1477,6 +1525,26 @@ const std::vector<double> &pw_cached(double alpha, const PwShape &sh, int np, in
     return it->second.tab;
 }
 
+// The fixed-point kernel's pair and correction tables at the scaled screening a,
+// one after the other.  The last kFxCached screenings are kept for the process (a
+// caller holds its table by the shared pointer).
+constexpr size_t kFxTableBytes = sizeof(FxRow) * (kFxOctaves * kFxSub + kFxCorrRows);
+constexpr size_t kFxCached = 16;
+std::shared_ptr<const std::vector<FxRow>> fx_cached(double a) {
+    static std::mutex mu;
+    static std::vector<std::pair<double, std::shared_ptr<const std::vector<FxRow>>>> cache;
+    std::lock_guard<std::mutex> lock(mu);
+    for (auto &c : cache)
+        if (c.first == a) return c.second;
+    auto pair = std::make_shared<std::vector<FxRow>>();
+    std::vector<FxRow> corr;
+    fx_build_tables(a, *pair, corr);
+    pair->insert(pair->end(), corr.begin(), corr.end());
+    if (cache.size() >= kFxCached) cache.erase(cache.begin());
+    cache.emplace_back(a, pair);
+    return pair;
+}
+
 // The kernel's table evaluation on the host (same bit indexing, same fused
 // Horner steps), for the host-only diagnostic.
 bool pw_eval_host(const PwShape &sh, const double *tab, int npieces, double arg, double &f,
@@ -1710,17 +1778,29 @@ int apply_t(qeq_ctx *ctx, const double *R, const double *q, const double *sigma,
     T *sg = f64 ? (T *)ctx->sg64 : (T *)ctx->sg32;
     const qeq_params &p = ctx->p;
     ctx->applies++;
+    // FP64 real space: fixed point where its tile fits a block (k_real64 otherwise).
+    // The tile capacity changes only in a neighbour build, after which every array
+    // is gathered again.
+    const FxLaunch fl64 = f64 ? fx_launch(ctx) : FxLaunch{};
+    FxGather fx{};
+    if (fl64.on) {
+        fx.x = ctx->xfix;
+        fx.s2 = ctx->sfix;
+        fx.coord_bits = kFxCoordBits - ctx->fx_exp;
+        fx.sigma_bits = kFxSigmaBits - 2 * ctx->fx_exp;
+    }
     prof_begin(ctx, kPhGatherIn, s);
     if (q_only) {
-        k_gather_q<T><<<grid_for(n), kThreads, 0, s>>>(n, ctx->perm, q, xq, (T4 *)ctx->sfrac,
+        k_gather_q<T><<<grid_for(n), kThreads, 0, s>>>(n, ctx->perm, q, xq, (T4 *)ctx->sfrac, fx,
                                                        ctx->d_flags);
     } else {
-        int32_t *smax_bits = (!f64 && kRealLazySigma) ? ctx->d_flags + kFlagSigmaMax : nullptr;
+        int32_t *smax_bits =
+            (f64 ? fl64.on : kRealLazySigma) ? ctx->d_flags + kFlagSigmaMax : nullptr;
         if (smax_bits) cudaMemsetAsync(smax_bits, 0, sizeof(int32_t), s);
         k_gather_in<T><<<grid_for(n), kThreads, 0, s>>>(
             n, ctx->perm, R, ctx->wrap_off, q, sigma, ctx->K[0] / p.box[0], ctx->K[1] / p.box[1],
             ctx->K[2] / p.box[2], xq, sg, ctx->sbase, (T4 *)ctx->sfrac, smax_bits,
-            f64 ? ctx->xf_pre : nullptr, ctx->d_flags);
+            f64 && !fl64.on ? ctx->xf_pre : nullptr, fx, ctx->d_flags);
         ctx->gathered = true;
     }
     prof_end(ctx, s);
@@ -1775,7 +1855,31 @@ int apply_t(qeq_ctx *ctx, const double *R, const double *q, const double *sigma,
         const dim3 grid((unsigned)ctx->geom.nbricks);
         int32_t *fl = ctx->d_flags;
         unsigned char *gt = ctx->tile_scratch;
-        if (f64) {
+        if (f64 && fl64.on) {
+            FxArgs fa{};
+            fa.nchunk = fl64.nchunk;
+            fa.tpr_log2 = fl64.tpr_log2;
+            fa.coord_bits = fx.coord_bits;
+            fa.sigma_bits = fx.sigma_bits;
+            fa.hi_cut = fl64.hi_cut;
+            for (int d = 0; d < 3; ++d) fa.L[d] = fx_from_double(p.box[d], fx.coord_bits);
+            fa.fx_exp = ctx->fx_exp;
+            fa.v_scale = std::ldexp(p.k_e, -ctx->fx_exp);
+            fa.e_scale = std::ldexp(p.k_e, -2 * ctx->fx_exp);
+            const FxExact fe{ra, (const double4_32a *)xq, (const double *)sg, ctx->erfc_tab64,
+                             (const double2 *)ctx->fg_tab64, (const double2 *)ctx->gc_tab64};
+            const FxRow *pt = (const FxRow *)ctx->fx_tab, *ct = pt + kFxOctaves * kFxSub;
+            const dim3 fgrid((unsigned)std::min<int64_t>(ctx->geom.nbricks * fl64.nchunk, ctx->sm_count));
+            auto launch = [&](auto kern) {
+                kern<<<fgrid, fl64.threads, fl64.smem, s>>>(
+                    fa, fe, ctx->geom, ctx->tile_tab, ctx->tile_tot, ctx->nbr, ctx->cnt, ctx->xfix,
+                    ctx->sfix, pt, fl64.npair, ct, ctx->tile_cap, fl64.qcap, fl, ctx->v_s, ctx->E_s);
+            };
+            if (need_field && fl64.corr_smem) launch(k_real64_fixed<true, true>);
+            else if (need_field) launch(k_real64_fixed<true, false>);
+            else if (fl64.corr_smem) launch(k_real64_fixed<false, true>);
+            else launch(k_real64_fixed<false, false>);
+        } else if (f64) {
             auto *x4 = (const double4_32a *)xq;
             auto *s1 = (const double *)sg;
             if (need_field && !L.gtile)
@@ -1808,6 +1912,7 @@ int apply_t(qeq_ctx *ctx, const double *R, const double *q, const double *sigma,
     if (!pme) {
         int rc = ewald_recip_and_combine(ctx, q, sigma, v, E, F, need_field, s);
         if (rc) return rc;
+        if (fl64.on) cudaMemsetAsync(ctx->d_flags + kFlagChargeExp, 0, sizeof(int32_t), s);
         if (energy4) {
             k_finalize<<<4, kThreads, 0, s>>>(ctx->part, ctx->red_grid, energy4);
             ctx->launches++;
@@ -1828,6 +1933,7 @@ int apply_t(qeq_ctx *ctx, const double *R, const double *q, const double *sigma,
     ga.sz_f = (float)ga.sz;
     ga.self_coef_f = (float)ga.self_coef;
     ga.gauss_coef_f = (float)ga.gauss_coef;
+    ga.charge_exp = fl64.on ? ctx->d_flags + kFlagChargeExp : nullptr;
     prof_begin(ctx, kPhGatherOut, s);
     const bool energy = energy4 != nullptr;
     if (need_field)
@@ -1905,6 +2011,11 @@ int coulomb_alloc(qeq_ctx *ctx) {
     ctx->mesh_n = (int64_t)ctx->K[0] * ctx->K[1] * ctx->K[2];
     ctx->meshc_n = (int64_t)ctx->K[0] * ctx->K[1] * K2h;
     const size_t rs = ctx->fp32 ? sizeof(float) : sizeof(double);
+    // Fixed-point real space in FP64 mode where the tile's coordinates stay inside
+    // half its range (16 scaled lengths): with r_cut' in (4, 8], any usual skin.
+    ctx->fx_exp = fx_exponent(p.r_cut);
+    ctx->fx_on = !ctx->fp32 && std::ldexp(p.r_cut + 2.0 * p.skin, -ctx->fx_exp) < 15.0 &&
+                 std::abs(ctx->fx_exp) < 400;
     struct {
         void **ptr;
         size_t bytes;
@@ -1916,6 +2027,9 @@ int coulomb_alloc(qeq_ctx *ctx) {
         {ctx->fp32 ? (void **)&ctx->xq32 : (void **)&ctx->xq64, 4 * rs * n},
         {ctx->fp32 ? (void **)&ctx->sg32 : (void **)&ctx->sg64, rs * n},
         {(void **)&ctx->xf_pre, ctx->fp32 ? 0 : sizeof(float4) * n},
+        {(void **)&ctx->xfix, ctx->fx_on ? sizeof(ulonglong4_32a) * n : 0},
+        {(void **)&ctx->sfix, ctx->fx_on ? sizeof(u64) * n : 0},
+        {(void **)&ctx->fx_tab, ctx->fx_on ? kFxTableBytes : 0},
         {&ctx->mesh, rs * ctx->mesh_n},
         {&ctx->meshc, 2 * rs * ctx->meshc_n},
         {&ctx->G, rs * ctx->meshc_n},
@@ -2003,6 +2117,10 @@ int coulomb_alloc(qeq_ctx *ctx) {
         if (ea == cudaSuccess)
             ea = cudaFuncSetAttribute(k_real64<false, true>,
                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kReal64SmemMax);
+        for (const void *k : {(const void *)k_real64_fixed<true, true>, (const void *)k_real64_fixed<true, false>,
+                              (const void *)k_real64_fixed<false, true>, (const void *)k_real64_fixed<false, false>})
+            if (ea == cudaSuccess)
+                ea = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kReal64SmemMax);
         const int rca = cuda_check(ctx, ea, "real-space shared memory attribute");
         if (rca) return rca;
     }
@@ -2042,6 +2160,14 @@ int coulomb_alloc(qeq_ctx *ctx) {
             rc = cuda_check(ctx, e, "pair-function table upload");
             if (rc) return rc;
         }
+    }
+
+    if (ctx->fx_on) {
+        // pageable memory: the copy has left it when the call returns
+        const auto tab = fx_cached(std::ldexp(p.alpha, ctx->fx_exp));
+        e = cudaMemcpyAsync(ctx->fx_tab, tab->data(), kFxTableBytes, cudaMemcpyHostToDevice, ctx->alloc_stream);
+        rc = cuda_check(ctx, e, "fixed-point table upload");
+        if (rc) return rc;
     }
 
     // cuFFT plans (from the plan pool) with a work area from this library's
@@ -2121,6 +2247,7 @@ void plan_release(int dev, const int K[3], cufftType type, cufftHandle h, size_t
 }
 
 int real_tile_reserve(qeq_ctx *ctx) {
+    if (fx_launch(ctx).on) return QEQ_OK;  // its tile is always in shared memory
     const RealLaunch L = real_launch(ctx, !ctx->fp32);
     if (!L.gtile) return QEQ_OK;
     const size_t need = (size_t)ctx->geom.nbricks * L.cap * (ctx->fp32 ? kTile32Bytes : kTile64Bytes);
@@ -2144,6 +2271,7 @@ void coulomb_free(qeq_ctx *ctx) {
     void *ptrs[] = {ctx->v_s,  ctx->E_s,  ctx->sbase, ctx->sfrac, ctx->xq32, ctx->xq64,
                     ctx->sg32, ctx->sg64, ctx->mesh,  ctx->meshc, ctx->G,    ctx->part,
                     ctx->scal, ctx->energy4, ctx->fft_work, ctx->erfc_tab64, ctx->fg_tab64, ctx->gc_tab64, ctx->xf_pre, ctx->tile_scratch,
+                    ctx->xfix, ctx->sfix, ctx->fx_tab,
                     ctx->ticket};
     for (void *p : ptrs) dev_free(ctx, p);
     if (ctx->pme_stream) side_release(ctx->device, ctx->pme_stream, ctx->pme_fork, ctx->pme_join);
@@ -2178,6 +2306,39 @@ int pair_table_eval_host(int which, double alpha, double smax, int64_t n, const 
             F[k] = f;
             G[k] = g;
         }
+    }
+    return QEQ_OK;
+}
+
+// One pair as the fixed-point kernel evaluates it, per unit charge, on the host.
+int fixed_pair_eval_host(double alpha, double r_cut, int64_t n, const double *d, const double *si,
+                         const double *sj, double *f, double *gc, int32_t *path) {
+    const int e = fx_exponent(r_cut);
+    const auto tab = fx_cached(std::ldexp(alpha, e));
+    const FxRow *pt = tab->data(), *ct = pt + kFxOctaves * kFxSub;
+    const double rc = std::ldexp(r_cut, -e);
+    const u32 hi_cut = (u32)std::floor(std::ldexp(rc * rc, 22)) - 1u;
+    for (int64_t k = 0; k < n; ++k) {
+        const u64 s = fx_dist2((s64)fx_from_double(d[3 * k], kFxCoordBits - e),
+                               (s64)fx_from_double(d[3 * k + 1], kFxCoordBits - e),
+                               (s64)fx_from_double(d[3 * k + 2], kFxCoordBits - e));
+        const u32 sh = fx_hi(s);
+        path[k] = -1;
+        if (sh > hi_cut + 2) continue;
+        const int lz = fx_clz(sh);
+        path[k] = 0;
+        if (sh >= hi_cut || lz > kFxLzMin) continue;
+        const u64 y = fx_pos(s, lz);
+        const int b = fx_bshift(lz);
+        u64 fu, gu;
+        fx_eval<true, kFxGShift>(pt[fx_piece(sh, lz)], fx_hi(y), fx_lo(y), fu, gu);
+        s64 F = (s64)fu, G = (s64)gu;
+        const u64 g2 = fx_sigma2(si[k], kFxSigmaBits - 2 * e) + fx_sigma2(sj[k], kFxSigmaBits - 2 * e);
+        const u32 gh = fx_hi(g2);
+        if ((sh >> 3) < gh + (gh >> 3) && !(g2 < kFxSigmaSat && fx_correct<true>(ct, s, b, g2, F, G))) continue;
+        path[k] = 1;
+        f[k] = std::ldexp((double)F, -kFxFBits - e);
+        gc[k] = -std::ldexp((double)G, b - kFxGBits - 3 * e);
     }
     return QEQ_OK;
 }

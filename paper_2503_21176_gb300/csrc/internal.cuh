@@ -58,7 +58,8 @@ constexpr double kSqrtTwoOverPi = 0.79788456080286535588;
 constexpr double kPi = 3.14159265358979323846;
 
 // Device-side status words (int32).
-// kFlagSigmaMax: float bits of max |sigma| of the last FP32 apply's inputs.
+// kFlagSigmaMax: float bits of max |sigma| of the last FP32 apply's inputs (FP64
+// fixed-point real space: the largest high word of the scaled sigma^2).
 // kFlagMaxTile / kFlagMaxRows: largest tile (atoms) and brick (rows) of the last build.
 // kFlagTileOverflow: a real-space block met a tile larger than its capacity
 // (cannot happen for a list built by this context; the block then skips its brick).
@@ -70,6 +71,9 @@ enum Flag {
     kFlagMaxRows = 4,
     kFlagTileOverflow = 5,
     kFlagBounds = 6,  // bounds-checked build: first failing check site (kept across builds)
+    // Largest biased exponent of the charges of the apply in progress (FP64
+    // fixed-point real space): raised by the gather, cleared at the apply's end.
+    kFlagChargeExp = 7,
     kNumFlags = 8
 };
 
@@ -352,6 +356,13 @@ struct qeq_ctx {
     double *gc_tab64 = nullptr;    // piecewise F_1(t), G_1(t) of the Gaussian correction (FP64)
     int gc_pieces = 0;
     float4 *xf_pre = nullptr;      // [N] FP32 positions (sorted) of the FP64 kernel's prefilter
+    // FP64 real space in fixed point (fixed64.cuh): used where fx_on; fx_exp is the
+    // exponent e of its scaled lengths r / 2^e.
+    bool fx_on = false;
+    int fx_exp = 0;
+    ulonglong4_32a *xfix = nullptr;  // [N] (x, y, z as coordinates, bits of q) (sorted)
+    uint64_t *sfix = nullptr;        // [N] scaled sigma^2 (sorted)
+    unsigned char *fx_tab = nullptr; // pair table, then correction table
 
     // ---- explicit k-vector Ewald (ewald.cu) ----
     void *ewald_k = nullptr;        // [nk] double4 (kx, ky, kz, g)
