@@ -439,6 +439,290 @@ k_emit(EmitArgs a, BrickGeom g, int nchunk, const double4_32a *__restrict__ xs64
     }
 }
 
+// The grouped form (small systems): rows a warp tests against each candidate (their
+// positions stay in registers), and its block.
+constexpr int kGroupRows = 4;
+constexpr int kGroupThreads = 256;
+// Systems below this many atoms per SM (38,912 on a 152-SM GB300) use it: there the
+// four-lane form leaves the chip idle and waits on its serial candidate loop.  Whole
+// builds, four lanes a row / grouped, r_list 9 A: 102 atoms 129 / 85 us, 648 153 / 92,
+// 3,000 202 / 117, 9,999 202 / 178, 20,001 319 / 319, 36,000 525 / 489, 60,000
+// 614 / 673, 300,000 1,622 / 2,548.
+constexpr int64_t kGroupAtomsPerSm = 256;
+
+// Candidate ranges of one cell, built by one warp: its (2 reach + 1)^3 neighbour
+// cells in order, empty ones dropped and those that continue one sorted range in the
+// same tile brick under the same image shift merged.  Entry k: (candidates up to and
+// including this range, first sorted atom less the candidates before the range, tile
+// base, image code).  tmp holds the cells before the merge.  Returns the number of
+// ranges (*total candidates).
+__device__ __forceinline__ int cell_ranges(const EmitArgs &a, const BrickGeom &g, int bx, int by, int bz,
+                                           int lc, const int32_t *__restrict__ cell_start,
+                                           const int *t_base, int4 *tmp, int4 *ranges, int *total) {
+    const int lane = threadIdx.x & 31;
+    const unsigned lt = (1u << lane) - 1u;
+    const int dy = 2 * a.ry + 1, dz = 2 * a.rz + 1, ncand = (2 * a.rx + 1) * dy * dz;
+    // Bricks are 1 or 2 cells per axis, so every division by B is a shift (lb =
+    // log2 B); the flat index splits by FP32 reciprocals (exact below 2^22); and
+    // with at least reach cells per axis a neighbour cell's image shift is -1, 0
+    // or 1 by comparison (fewer cells take the general floor division).
+    const int lb0 = g.B[0] - 1, lb1 = g.B[1] - 1, lb2 = g.B[2] - 1;
+    const bool near = a.ncx >= a.rx && a.ncy >= a.ry && a.ncz >= a.rz;
+    const float inv_yz = 1.0f / (float)(dy * dz), inv_z = 1.0f / (float)dz;
+    const int cx = (bx << lb0) + (lc >> (lb2 + lb1)), cy = (by << lb1) + ((lc >> lb2) & lb1),
+              cz = (bz << lb2) + (lc & lb2);
+    int m = 0;
+    for (int k0 = 0; k0 < ncand; k0 += 32) {
+        const int kk = k0 + lane;
+        int4 e = make_int4(0, 0, 0, 0);
+        if (kk < ncand) {
+            const int qx = __float2int_rz(((float)kk + 0.5f) * inv_yz), rem = kk - qx * (dy * dz);
+            const int qy = __float2int_rz(((float)rem + 0.5f) * inv_z);
+            const int ux = cx + qx - a.rx, uy = cy + qy - a.ry, uz = cz + (rem - qy * dz) - a.rz;
+            int sx, sy, sz;
+            if (near) {
+                sx = ux < 0 ? -1 : (ux >= a.ncx ? 1 : 0);
+                sy = uy < 0 ? -1 : (uy >= a.ncy ? 1 : 0);
+                sz = uz < 0 ? -1 : (uz >= a.ncz ? 1 : 0);
+            } else {
+                sx = floor_div(ux, a.ncx);
+                sy = floor_div(uy, a.ncy);
+                sz = floor_div(uz, a.ncz);
+            }
+            const int wx = ux - sx * a.ncx, wy = uy - sy * a.ncy, wz = uz - sz * a.ncz;
+            const int tx = (ux >> lb0) - bx + g.br[0];
+            const int ty = (uy >> lb1) - by + g.br[1];
+            const int tz = (uz >> lb2) - bz + g.br[2];
+            const int cn = (int)(brick_index(g, wx >> lb0, wy >> lb1, wz >> lb2) * g.bvol +
+                                 (((wx & lb0) << lb1 | (wy & lb1)) << lb2 | (wz & lb2)));
+            e = make_int4(cell_start[cn], cell_start[cn + 1], t_base[(tx * g.td[1] + ty) * g.td[2] + tz],
+                          (sx + 2) * 25 + (sy + 2) * 5 + (sz + 2));
+        }
+        const bool some = e.y > e.x;
+        const unsigned bal = __ballot_sync(0xffffffffu, some);
+        if (some) tmp[m + __popc(bal & lt)] = e;
+        m += __popc(bal);
+    }
+    __syncwarp();
+    int nr = 0, before = 0;  // ranges, and candidates before this round
+    for (int k0 = 0; k0 < m; k0 += 32) {
+        const int t = k0 + lane;
+        const bool in = t < m;
+        const int4 e = in ? tmp[t] : make_int4(0, 0, 0, 0);
+        const int4 pe = in && t > 0 ? tmp[t - 1] : make_int4(-1, -1, -1, -1);
+        const bool first = in && !(pe.y == e.x && pe.z == e.z && pe.w == e.w);
+        int x = e.y - e.x;  // inclusive scan of the cells' atoms
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        const unsigned bal = __ballot_sync(0xffffffffu, first);
+        const int upto = before + x, start = upto - (e.y - e.x);
+        if (first) {
+            const int r = nr + __popc(bal & lt);
+            if (r > 0) ranges[r - 1].x = start;
+            ranges[r].y = e.x - start;
+            ranges[r].z = e.z;
+            ranges[r].w = e.w;
+        }
+        nr += __popc(bal);
+        before += __shfl_sync(0xffffffffu, x, 31);
+        __syncwarp();
+    }
+    if (lane == 0) {
+        if (nr > 0) ranges[nr - 1].x = before;
+        *total = before;
+    }
+    return nr;
+}
+
+// One block per brick, or nchunk blocks (each takes the brick's row groups c,
+// c + nchunk, ...).  Warp 0 builds the tile table, then each warp the candidate
+// ranges of a cell.  A warp then takes a group of up to kGroupRows rows of one cell:
+// its lanes walk the cell's candidates 32 at a time, each lane holding one candidate
+// against which all rows of the group are tested, and ballots count a row's kept
+// candidates per distance class.  A second walk repeats the tests and writes every
+// kept candidate at its place (class order, candidates in order inside a class).
+// The decision is FP32 outside the band [lo, hi] and FP64 inside (band_keep); the
+// class comes from the FP32 d^2.  The block also records the largest tile and brick
+// for the real-space launch, and writes no entry when the tile exceeds 16-bit indices.
+//
+__global__ void __launch_bounds__(kGroupThreads)
+k_emit_group(const __grid_constant__ EmitArgs a, const __grid_constant__ BrickGeom g, int nchunk, int rows_per_group,
+       const double4_32a *__restrict__ xs64, const float4 *__restrict__ xs32,
+       const int32_t *__restrict__ cell_start, uint16_t *__restrict__ nbr, int32_t *__restrict__ cnt,
+       int4 *__restrict__ tile_tab, int32_t *__restrict__ tile_tot, int32_t *__restrict__ flags) {
+    constexpr int NW = kGroupThreads / 32;
+    __shared__ int t_start[kMaxTileBricks], t_base[kMaxTileBricks], t_code[kMaxTileBricks], t_total;
+    __shared__ int4 tmp[NW][kMaxTileBricks];
+    __shared__ int4 ranges[kMaxBrickCells][kMaxTileBricks];
+    __shared__ float4 shtab[kMaxTileBricks];  // image shift s L of each code (sx + 2) * 25 + ...
+    __shared__ int ncand[kMaxBrickCells];
+    const int64_t b = blockIdx.x / nchunk;
+    const int chunk = (int)(blockIdx.x - b * nchunk);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (warp == 0) tile_table(g, b, cell_start, t_start, t_base, t_code, &t_total);
+    for (int code = threadIdx.x; code < 125; code += kGroupThreads)
+        shtab[code] = make_float4((float)(code / 25 - 2) * a.Lfx, (float)((code / 5) % 5 - 2) * a.Lfy,
+                                  (float)(code % 5 - 2) * a.Lfz, 0.f);
+    __syncthreads();
+    const int i0 = t_start[g.center], i1 = cell_start[(b + 1) * g.bvol];
+    if (chunk == 0) {
+        // the tile table of the brick, for the real-space kernels of this list
+        for (int rb = threadIdx.x; rb < g.T; rb += kGroupThreads)
+            tile_tab[b * g.T + rb] = make_int4(t_start[rb], t_base[rb], t_code[rb], 0);
+        if (threadIdx.x == 0) {
+            tile_tot[b] = t_total;
+            atomicMax(&flags[kFlagMaxTile], t_total);
+            atomicMax(&flags[kFlagMaxRows], i1 - i0);
+        }
+    }
+    if (t_total > kMaxTileAtoms) {
+        if (chunk == 0)
+            for (int i = i0 + threadIdx.x; i < i1; i += kGroupThreads) cnt[i] = 0;
+        return;
+    }
+    const int bz = (int)(b % g.nb[2]), by = (int)((b / g.nb[2]) % g.nb[1]);
+    const int bx = (int)(b / ((int64_t)g.nb[2] * g.nb[1]));
+    for (int lc = warp; lc < g.bvol; lc += NW)
+        cell_ranges(a, g, bx, by, bz, lc, cell_start, t_base, tmp[warp], ranges[lc], &ncand[lc]);
+    __syncthreads();
+    const unsigned lt = (1u << lane) - 1u;
+    const size_t stripe = (size_t)a.n * kListStripe;
+    // this warp's groups, counted through the brick's cells
+    int next = chunk * NW + warp, seen = 0;
+    for (int lc = 0; lc < g.bvol; ++lc) {
+        const int c0 = cell_start[b * g.bvol + lc], cn = cell_start[b * g.bvol + lc + 1] - c0;
+        const int ng = (cn + rows_per_group - 1) / rows_per_group;
+        for (; next < seen + ng; next += nchunk * NW) {
+            // the cell's rows split evenly over its groups
+            const int gi = next - seen;
+            const int rb = c0 + (int)((int64_t)cn * gi / ng), re = c0 + (int)((int64_t)cn * (gi + 1) / ng);
+            const int nr = re - rb;
+            float px[kGroupRows], py[kGroupRows], pz[kGroupRows];
+#pragma unroll
+            for (int r = 0; r < kGroupRows; ++r) {
+                const float4 x = xs32[rb + min(r, nr - 1)];
+                px[r] = x.x;
+                py[r] = x.y;
+                pz[r] = x.z;
+            }
+            const int4 *rt = ranges[lc];
+            const int total = ncand[lc];
+            // The group's candidates, 32 at a time: use(d^2 of each row, the rows that
+            // drop the candidate (bit r), its tile entry).  Dropped are, besides those
+            // beyond the band: the row itself (home image) and the pairs inside the band
+            // that the exact decision drops.
+            auto walk = [&](auto &&use) {
+                int k = 0;
+                for (int p0 = 0; p0 < total; p0 += 32) {
+                    const int p = p0 + lane;
+                    float xj = 1e18f, yj = 1e18f, zj = 1e18f;  // far: no row keeps it
+                    int j = -1, code = 0, ebase = 0;
+                    if (p < total) {
+                        int4 e = rt[k];
+                        while (p >= e.x) e = rt[++k];
+                        j = p + e.y;
+                        code = e.w;
+                        ebase = e.z;
+                        const float4 x = xs32[j];
+                        const float4 sh = shtab[code];
+                        xj = x.x + sh.x;
+                        yj = x.y + sh.y;
+                        zj = x.z + sh.z;
+                    }
+                    float d2[kGroupRows];
+                    bool band = false;
+#pragma unroll
+                    for (int r = 0; r < kGroupRows; ++r) {
+                        if (r >= nr) break;
+                        const float dx = xj - px[r], dy = yj - py[r], dz = zj - pz[r];
+                        d2[r] = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
+                        band = band || (d2[r] <= a.hi && !(d2[r] < a.lo));
+                    }
+                    const unsigned self = (unsigned)(j - rb);
+                    unsigned drop = code == kCenterCode && self < (unsigned)nr ? 1u << self : 0u;
+                    if (band) {
+#pragma unroll
+                        for (int r = 0; r < kGroupRows; ++r)
+                            if (r < nr && d2[r] <= a.hi && !(d2[r] < a.lo) &&
+                                !band_keep(&a, code, xs64 + j, xs64 + rb + r))
+                                drop |= 1u << r;
+                    }
+                    use(d2, drop, j + ebase);
+                }
+            };
+            // first walk: each lane counts its candidates per row and class
+            int all[kGroupRows], nc[kGroupRows];  // kept; near | inside the cutoff << 16
+#pragma unroll
+            for (int r = 0; r < kGroupRows; ++r) all[r] = nc[r] = 0;
+            walk([&](const float (&d2)[kGroupRows], unsigned drop, int) {
+#pragma unroll
+                for (int r = 0; r < kGroupRows; ++r) {
+                    if (r >= nr) break;
+                    all[r] += d2[r] <= a.hi ? 1 : 0;
+                    nc[r] += d2[r] < a.t_cut ? 0x10000 : 0;
+                    nc[r] += d2[r] < a.t_near ? 1 : 0;
+                }
+                if (drop) {
+#pragma unroll
+                    for (int r = 0; r < kGroupRows; ++r)
+                        if (r < nr && drop >> r & 1u) {
+                            all[r] -= 1;
+                            nc[r] -= (d2[r] < a.t_cut ? 0x10000 : 0) + (d2[r] < a.t_near ? 1 : 0);
+                        }
+                }
+            });
+            // counts to first slots; rows that do not fit are reported and not written
+            int near[kGroupRows], cut[kGroupRows];
+            bool over = false;
+#pragma unroll
+            for (int r = 0; r < kGroupRows; ++r) {
+                if (r >= nr) break;
+                const int tot = __reduce_add_sync(0xffffffffu, all[r]);
+                near[r] = 0;
+                cut[r] = __reduce_add_sync(0xffffffffu, nc[r] & 0xffff);
+                all[r] = __reduce_add_sync(0xffffffffu, nc[r] >> 16);
+                const bool fits = tot <= a.width;
+                if (lane == 0) {
+                    cnt[rb + r] = fits ? tot : 0;
+                    if (!fits) atomicMax(&flags[kFlagMaxRow], tot);
+                }
+                over = over || !fits;
+                if (fits) {  // pad to the stripe end with the tile's far sentinel slot
+                    const int pad = (tot + kListStripe - 1) / kListStripe * kListStripe;
+                    if (tot + lane < pad) nbr[list_index(tot + lane, rb + r, a.n)] = (uint16_t)t_total;
+                }
+            }
+            if (over) continue;  // the list is rebuilt with wider rows
+            walk([&](const float (&d2)[kGroupRows], unsigned drop, int e) {
+#pragma unroll
+                for (int r = 0; r < kGroupRows; ++r) {
+                    if (r >= nr) break;
+                    const bool keep = d2[r] <= a.hi && !(drop >> r & 1u);
+                    const unsigned m = __ballot_sync(0xffffffffu, keep);
+                    if (m == 0) continue;
+                    const bool c1 = d2[r] < a.t_cut, c0n = d2[r] < a.t_near;
+                    const unsigned mn = __ballot_sync(0xffffffffu, c0n) & m;
+                    const unsigned mc = __ballot_sync(0xffffffffu, c1) & m & ~mn;
+                    const unsigned ms = m & ~(mc | mn);
+                    if (keep && QEQ_IN_BOUNDS((unsigned)e < (unsigned)t_total, flags, kSiteEmitTile)) {
+                        const int slot = (c0n ? near[r] : c1 ? cut[r] : all[r]) +
+                                         __popc((c0n ? mn : c1 ? mc : ms) & lt);
+                        nbr[(slot >> 4) * stripe + (size_t)(rb + r) * kListStripe + (slot & 3) * 4 +
+                            ((slot >> 2) & 3)] = (uint16_t)e;
+                    }
+                    near[r] += __popc(mn);
+                    cut[r] += __popc(mc);
+                    all[r] += __popc(ms);
+                }
+            });
+        }
+        seen += ng;
+    }
+}
+
 // Per-atom search (qeq_set_neighbor_method QEQ_NL_ATOM): the form of the paper's
 // Triton neighbour kernel (Sec. 3.1), one thread per atom looping over the
 // cells around its own, written in this library's list format so that the
@@ -670,14 +954,17 @@ int nl_alloc_list(qeq_ctx *ctx, int width) {
     ctx->nbr_scratch = nullptr;
     int rc = dev_alloc(ctx, (void **)&ctx->nbr, sizeof(uint16_t) * (size_t)width * ctx->n);
     if (rc) return rc;
-    rc = dev_alloc(ctx, (void **)&ctx->nbr_scratch, sizeof(uint32_t) * (size_t)width * ctx->n);
-    if (rc) return rc;
+    if (!ctx->emit_group) {
+        rc = dev_alloc(ctx, (void **)&ctx->nbr_scratch, sizeof(uint32_t) * (size_t)width * ctx->n);
+        if (rc) return rc;
+    }
     ctx->width = width;
     return QEQ_OK;
 }
 
 int nl_alloc(qeq_ctx *ctx) {
     const int64_t n = ctx->n;
+    ctx->emit_group = n < kGroupAtomsPerSm * ctx->sm_count;
     struct {
         void **ptr;
         size_t bytes;
@@ -748,6 +1035,24 @@ static int launch_emit(qeq_ctx *ctx, cudaStream_t s) {
             a, ctx->geom, ctx->xs64, ctx->xs32, ctx->cell_s, ctx->cell_start, ctx->tile_tab,
             ctx->tile_tot, ctx->nbr, ctx->cnt, ctx->d_flags);
         return 2;
+    }
+    if (ctx->emit_group) {
+        // rows per group: as many as leave about eight groups an SM; blocks per brick:
+        // one per eight groups of the largest brick (from the previous build; 1.5 x the
+        // mean before the first), at most about four blocks an SM
+        const int64_t nb = ctx->geom.nbricks;
+        const int rows = ctx->max_rows > 0 ? ctx->max_rows
+                                           : (int)std::ceil(1.5 * (double)ctx->n / (double)nb);
+        const int rpg = (int)std::max<int64_t>(
+            1, std::min<int64_t>(kGroupRows, ctx->n / (8 * (int64_t)ctx->sm_count)));
+        const int64_t groups = std::max<int64_t>(1, (rows + rpg - 1) / rpg);
+        const int nchunk = (int)std::max<int64_t>(
+            1, std::min<int64_t>((groups + kGroupThreads / 32 - 1) / (kGroupThreads / 32),
+                                 (4 * (int64_t)ctx->sm_count + nb - 1) / nb));
+        k_emit_group<<<(unsigned)(nb * nchunk), kGroupThreads, 0, s>>>(
+            a, ctx->geom, nchunk, rpg, ctx->xs64, ctx->xs32, ctx->cell_start, ctx->nbr, ctx->cnt,
+            ctx->tile_tab, ctx->tile_tot, ctx->d_flags);
+        return 1;
     }
     // blocks per brick: enough to put about kEmitBlocksPerSm blocks on every SM
     // when the box has few bricks, at most one per 32 rows of the largest brick
