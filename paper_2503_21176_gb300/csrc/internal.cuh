@@ -529,8 +529,12 @@ __device__ __forceinline__ double warp_max(double v) {
 // Programmatic dependent launch (sm_90 and later).  A kernel launched by
 // launch_pdl may be scheduled while the kernel before it on the stream is still
 // running; pdl_begin() then holds every thread until that kernel has completed
-// and its writes are visible, and lets the next kernel launch in turn.  Each such
-// kernel calls it first, before any access to memory; without the launch
+// and its writes are visible.  Each such kernel calls it first, before any access
+// to memory, and lets its own successor launch with pdl_end() when its loop over
+// the atoms is done and the block reductions remain: triggered at the start, the
+// successor's waiting blocks took SM slots that blocks of the running kernels
+// still needed (10 to 16 steps of 300,000 atoms queued back to back: 14.59 ms
+// against 13.7; the same steps one at a time 13.88).  Without the launch
 // attribute both instructions do nothing.  Inside a captured graph the
 // dependency becomes a programmatic edge.  The shadow-step kernels use it (a
 // chain of short grid-stride kernels: about 0.9 us per boundary) when their
@@ -540,10 +544,8 @@ __device__ __forceinline__ double warp_max(double v) {
 // real-space kernel, do not use it (the step graph ran 85 us slower), nor do
 // the members of a batched step, whose evaluations are parallel branches of
 // one graph (FP64 serving steps ran 5% slower).
-__device__ __forceinline__ void pdl_begin() {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
+__device__ __forceinline__ void pdl_begin() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_end() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 #ifndef QEQ_PDL
 #define QEQ_PDL 1  // 0: the same kernels launched without the attribute

@@ -73,6 +73,7 @@ __global__ void k_lambda_part(int n, double q_tot, const double *__restrict__ ch
         s1 += (chi[i] + v[i]) * iu;
         s2 += iu;
     }
+    pdl_end();
     double vals[2] = {s1, s2};
     block_sum<2>(vals);
     if (threadIdx.x == 0) {
@@ -104,6 +105,7 @@ __global__ void k_charges(int n, double q_tot, const double *__restrict__ chi,
         a[4] += nn[i] * v[i];
         a[5] += qi;
     }
+    pdl_end();
     block_sum<6>(a);
     if (threadIdx.x == 0)
         for (int k = 0; k < 6; ++k) part[k * kRedBlocks + blockIdx.x] = a[k];
@@ -137,6 +139,7 @@ __global__ void k_forces_w1(int n, const double *__restrict__ q, const double *_
         phi[i] = pw;
         s += pw * inv_u[i];
     }
+    pdl_end();
     double vals[1] = {s};
     block_sum<1>(vals);
     if (threadIdx.x == 0) part[blockIdx.x] = vals[0];
@@ -151,6 +154,7 @@ __global__ void k_mu_part(int n, const double *__restrict__ phi, const double *_
     double s = 0.0;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
         s += phi[i] * inv_u[i];
+    pdl_end();
     double vals[1] = {s};
     block_sum<1>(vals);
     if (threadIdx.x == 0) part[blockIdx.x] = vals[0];
@@ -177,6 +181,7 @@ __global__ void k_jacobian(int n, const double *__restrict__ phi, const double *
             s += w0[i] * ri;
         }
     }
+    pdl_end();
     if (wnext) {
         double vals[1] = {s};
         block_sum<1>(vals);
@@ -197,6 +202,7 @@ __global__ void k_axpy_dot(int n, const double *__restrict__ scal, const double 
         x[i] = xi;
         s += z[i] * xi;
     }
+    pdl_end();
     double vals[1] = {s};
     block_sum<1>(vals);
     if (threadIdx.x == 0) part[blockIdx.x] = vals[0];
@@ -212,6 +218,7 @@ __global__ void k_normalize(int n, const double *__restrict__ scal, double *__re
     const double inv = scal[S_INVN];
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
         x[i] *= inv;
+    pdl_end();
 }
 
 // One block: sum the partials of O = R^T R and g = R^T f in fixed order, solve
@@ -316,6 +323,7 @@ __global__ void k_normal_part(int n, const double *__restrict__ Rb, const double
 #pragma unroll
         for (int a = 0; a < M; ++a) acc[nO + a] += r[a] * fi;
     }
+    pdl_end();
     block_sum<nO + M>(acc);
     if (threadIdx.x == 0)
 #pragma unroll
@@ -365,6 +373,7 @@ __global__ void k_ls_residual(int n, int m, const double *__restrict__ Rb,
         for (int a = 0; a < m; ++a) r += c[a] * Rb[(size_t)a * n + i];
         acc += r * r;
     }
+    pdl_end();
     double vals[1] = {acc};
     block_sum<1>(vals);
     if (threadIdx.x == 0) part[blockIdx.x] = vals[0];
@@ -453,6 +462,7 @@ __global__ void k_advance(int n, double dt, double half_dt, double mass_unit, Di
         for (int k = dis.kd; k >= 1; --k) hist[(size_t)k * n + i] = h[k - 1];
         hist[i] = nn;
     }
+    pdl_end();
     max_last_block(f32_to_f64_exact(mx), part, max_d2, ticket);
 }
 
@@ -485,6 +495,7 @@ __global__ void k_finish(int n, double half_mass_unit, bool kick,
         }
         ke = fma(half_mass_unit * mass[i], v2, ke);
     }
+    pdl_end();
     double vals[1] = {ke};
     block_sum<1>(vals);
     if (threadIdx.x == 0) part[blockIdx.x] = vals[0];
