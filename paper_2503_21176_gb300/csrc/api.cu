@@ -361,9 +361,12 @@ bool step_graphable(const qeq_ctx *ctx, cudaStream_t s) {
 
 
 int ensure_step_graph(qeq_ctx *ctx, const qeq_md_params *prm, qeq_md_state *st, cudaStream_t s) {
+    // steps keep their pair values (a context that only evaluates does not pay for the
+    // memory); before the capture
+    if (step_keeps_pairs(ctx)) pair_reserve(ctx, s);
     const void *key[14] = {st->R, st->V, st->F, st->Kf, st->n_hist, st->q, st->energies,
                            prm->chi, prm->eta, prm->sigma, prm->mass, ctx->nbr, ctx->tile_scratch,
-                           nullptr};
+                           ctx->pair_f};
     bool same = ctx->step_exec && ctx->graph_width == ctx->width &&
                 ctx->graph_tile == ctx->tile_cap && ctx->graph_rows == ctx->rows_cap &&
                 ctx->graph_pdl == ctx->pdl;
@@ -415,6 +418,7 @@ void count_step_replay(qeq_ctx *ctx) {
 static int evaluate_and_finish(qeq_ctx *ctx, const qeq_md_params *prm, qeq_md_state *st,
                                cudaStream_t s) {
     if (!step_graphable(ctx, s)) {
+        if (step_keeps_pairs(ctx)) pair_reserve(ctx, s);
         int rc = shadow_evaluate(ctx, prm, st, s);
         if (rc) return rc;
         return shadow_finish(ctx, prm, st, true, s, true);

@@ -100,7 +100,7 @@ __global__ void k_gather_in(int n, const int32_t *__restrict__ perm, const doubl
                             typename V4<T>::type *__restrict__ xq, T *__restrict__ sg,
                             int4 *__restrict__ sbase, typename V4<T>::type *__restrict__ sfrac,
                             int32_t *__restrict__ smax_bits, float4 *__restrict__ xf, FxGather fx,
-                            int32_t *__restrict__ flags) {
+                            T *__restrict__ qs, int32_t *__restrict__ flags) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if constexpr (std::is_same<T, double>::value) {
         if (fx.x) {
@@ -126,6 +126,7 @@ __global__ void k_gather_in(int n, const int32_t *__restrict__ perm, const doubl
     const double y = R[3 * (size_t)a + 1] + w[3 * (size_t)a + 1];
     const double z = R[3 * (size_t)a + 2] + w[3 * (size_t)a + 2];
     const double qa = q[a];
+    if constexpr (std::is_same<T, double>::value) qs[i] = qa;
     // scaled fractional coordinates u = K x / L (x wrapped into [0, L)), split
     // into floor and fraction
     const double ux = x * sK0, uy = y * sK1, uz = z * sK2;
@@ -133,6 +134,7 @@ __global__ void k_gather_in(int n, const int32_t *__restrict__ perm, const doubl
         // FP32 copies truncated on the integer pipe (at most 1 ulp, against the
         // half ulp of rounding), the split exact from the bits
         const float qf = f64_to_f32_trunc(qa);
+        qs[i] = qf;
         xq[i] = {f64_to_f32_trunc(x), f64_to_f32_trunc(y), f64_to_f32_trunc(z), qf};
         sg[i] = f64_to_f32_trunc(sigma[a]);
         int kx, ky, kz;
@@ -166,7 +168,7 @@ template <typename T>
 __global__ void k_gather_q(int n, const int32_t *__restrict__ perm, const double *__restrict__ q,
                            typename V4<T>::type *__restrict__ xq,
                            typename V4<T>::type *__restrict__ sfrac, FxGather fx,
-                           int32_t *__restrict__ flags) {
+                           T *__restrict__ qs, int32_t *__restrict__ flags) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const bool in = i < n && QEQ_IN_BOUNDS((unsigned)perm[i] < (unsigned)n, flags, kSiteGatherPerm);
     T qa = T(0);
@@ -180,6 +182,7 @@ __global__ void k_gather_q(int n, const int32_t *__restrict__ perm, const double
         }
     }
     if (!in) return;
+    qs[i] = qa;
     xq[i].w = qa;
     sfrac[i].w = qa;
 }
@@ -316,6 +319,7 @@ constexpr size_t kTile32Bytes = 20, kTile64Bytes = 56;
 constexpr size_t kSmemPerBlock = 232448;
 constexpr size_t kReal32SmemMax = kSmemPerBlock - 4096;
 constexpr size_t kReal64SmemMax = kSmemPerBlock - 4096;  // tables included
+constexpr size_t kPairSmemMax = kSmemPerBlock - 4096;  // k_pair_sum's charges
 // Largest deferred Gaussian-correction queue of the FP64 kernel (entries per lane).
 constexpr int kCorrQueueMax = 48;
 
@@ -673,9 +677,10 @@ __device__ __forceinline__ void kahan_add(float &sum, float &comp, float x) {
 // the running chunk sums.  The correction is evaluated only when r^2 is below
 // the row's bound gpre = 25 (sigma_i^2 + max sigma^2) (x 1.0001 against
 // rounding), the only pairs where it can be kept; sigma_j is read there only.
-// c1 = -alpha^2 log2 e, so exp(-alpha^2 r^2) = 2^(c1 r^2).
+// c1 = -alpha^2 log2 e, so exp(-alpha^2 r^2) = 2^(c1 r^2).  Returns the pair value
+// (0 beyond the cutoff).
 template <bool FIELD>
-__device__ __forceinline__ void pair32(float dx, float dy, float dz, float qj, const float *sgj,
+__device__ __forceinline__ float pair32(float dx, float dy, float dz, float qj, const float *sgj,
                                        float si2, float gpre, float pal, float c1, float rc2,
                                        float tspa, float &vf, float &exf, float &eyf, float &ezf) {
     const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
@@ -707,7 +712,9 @@ __device__ __forceinline__ void pair32(float dx, float dy, float dz, float qj, c
             eyf = fmaf(gq, dy, eyf);
             ezf = fmaf(gq, dz, ezf);
         }
+        return f;
     }
+    return 0.f;
 }
 
 
@@ -717,14 +724,15 @@ __device__ __forceinline__ void pair32(float dx, float dy, float dz, float qj, c
 // the field term, FP32 sums (each lane about r_list^3 rho / 4 terms) and an FP32
 // shuffle combine of the lanes; the row's sums, scaled by k_e, go out as one
 // float4 (v, E) per sorted atom.  smax_bits holds the float bits of max |sigma|
-// over the atoms (written by the gather of the same apply).
-template <bool FIELD, bool GTILE>
+// over the atoms (written by the gather of the same apply).  KEEP: the pair values
+// go out too, four entries to a 16-byte store, for k_pair_sum.
+template <bool FIELD, bool GTILE, bool KEEP>
 __global__ void __launch_bounds__(kRealMaxThreads, QEQ_REAL_MIN_BLOCKS)
 k_real32(RealArgs a, BrickGeom g, const int4 *__restrict__ tile_tab, const int32_t *__restrict__ tile_tot,
          const uint16_t *__restrict__ nbr, const int32_t *__restrict__ cnt,
          const float4 *__restrict__ xq, const float *__restrict__ sg,
          const int32_t *__restrict__ smax_bits, int cap, unsigned char *__restrict__ gtile,
-         int32_t *__restrict__ flags, float4 *__restrict__ vE) {
+         int32_t *__restrict__ flags, float4 *__restrict__ vE, float *__restrict__ pair_f) {
     extern __shared__ __align__(32) unsigned char smem_raw[];
     __shared__ int t_start[kMaxTileBricks], t_base[kMaxTileBricks], t_code[kMaxTileBricks], t_total;
     unsigned char *base = GTILE ? gtile + (size_t)blockIdx.x * cap * kTile32Bytes : smem_raw;
@@ -757,6 +765,7 @@ k_real32(RealArgs a, BrickGeom g, const int4 *__restrict__ tile_tab, const int32
             const uint2 *pw = (const uint2 *)(nbr + list_index(sub, i, a.n));
             uint2 w0 = cl > 0 ? __ldg(pw) : make_uint2(0u, 0u);
             uint2 w1 = cl > 4 ? __ldg(pw + wstep) : make_uint2(0u, 0u);
+            float4 *pf = KEEP ? (float4 *)pair_f + list_index(sub, i, a.n) / 4 : nullptr;
             for (int t = 0; t < cl; t += 4) {
                 const uint2 cur = w0;
                 w0 = w1;
@@ -764,14 +773,19 @@ k_real32(RealArgs a, BrickGeom g, const int4 *__restrict__ tile_tab, const int32
                 w1 = t + 8 < cl ? __ldg(pw + wstep) : make_uint2(0u, 0u);
                 const int ev[4] = {(int)(cur.x & 0xffffu), (int)(cur.x >> 16), (int)(cur.y & 0xffffu),
                                    (int)(cur.y >> 16)};
+                float f[4] = {0.f, 0.f, 0.f, 0.f};
                 // entries past the row's end are padding (the far sentinel slot)
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
                     const int e = ev[u];
                     if (!QEQ_IN_BOUNDS(e <= total, flags, kSiteReal32Entry)) continue;
                     const float4 xc = tile[e];
-                    pair32<FIELD>(xc.x - xi.x, xc.y - xi.y, xc.z - xi.z, xc.w, tsg + e, si2, gpre,
-                                  a.pal_f, a.c1_f, a.rc2_f, a.tspa_f, tv, tx, ty, tz);
+                    f[u] = pair32<FIELD>(xc.x - xi.x, xc.y - xi.y, xc.z - xi.z, xc.w, tsg + e, si2, gpre,
+                                         a.pal_f, a.c1_f, a.rc2_f, a.tspa_f, tv, tx, ty, tz);
+                }
+                if (KEEP) {
+                    *pf = make_float4(f[0], f[1], f[2], f[3]);
+                    pf += wstep;
                 }
             }
         }
@@ -793,6 +807,76 @@ k_real32(RealArgs a, BrickGeom g, const int4 *__restrict__ tile_tab, const int32
             else
                 reinterpret_cast<float *>(vE)[4 * (size_t)i] = a.ke_f * tv;
         }
+    }
+}
+
+// Potential-only real space from kept pair values: v_i = scale sum f_ij q_j, one block
+// per brick, its tile's charges in shared memory, kTPR lanes per row.  It adds the
+// terms as the kernel that kept them does (FP32-mixed: the same result bit for bit).
+// Bound: the streams of the list (2 bytes an entry) and of the values (4 or 8): 552 MB
+// at 300,000 atoms in FP32, 111 us (0.75 of the measured copy bandwidth) against the
+// 150 us of k_real32; in FP64 a solve of 20,001 atoms 22.5 -> 17.3 ms.
+template <typename T>
+__global__ void __launch_bounds__(kRealMaxThreads)
+k_pair_sum(int n, BrickGeom g, const int4 *__restrict__ tile_tab, const int32_t *__restrict__ tile_tot,
+           const uint16_t *__restrict__ nbr, const int32_t *__restrict__ cnt, const T *__restrict__ qs,
+           const T *__restrict__ pair_f, T scale, int cap, int32_t *__restrict__ flags,
+           T *__restrict__ v, int vstride) {
+    extern __shared__ __align__(32) unsigned char smem_raw[];
+    __shared__ int t_start[kMaxTileBricks], t_base[kMaxTileBricks], t_total;
+    T *tq = (T *)smem_raw;
+    for (int rb = threadIdx.x; rb < g.T; rb += blockDim.x) {
+        const int4 e = tile_tab[(int64_t)blockIdx.x * g.T + rb];
+        t_start[rb] = e.x;
+        t_base[rb] = e.y;
+    }
+    if (threadIdx.x == 0) t_total = tile_tot[blockIdx.x];
+    __syncthreads();
+    const int total = t_total;
+    if (total + 1 > cap) {
+        if (threadIdx.x == 0) atomicExch(&flags[kFlagTileOverflow], 1);
+        return;
+    }
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    for (int rb = warp; rb < g.T; rb += nw) {
+        const int st = t_start[rb], off = st + t_base[rb];
+        const int end = rb + 1 < g.T ? t_start[rb + 1] + t_base[rb + 1] : total;
+        for (int k = lane; k < end - off; k += 32) tq[off + k] = qs[st + k];
+    }
+    if (threadIdx.x == 0) tq[total] = T(0);  // the padding entries' slot
+    __syncthreads();
+    int i0, offc, nrows;
+    home_rows(g, t_start, t_base, total, i0, offc, nrows);
+    const size_t wstep = (size_t)kListStripe / 4 * n;  // one stripe further, in words of four entries
+    const int rpp = blockDim.x / kTPR;
+    for (int r0 = 0; r0 < nrows; r0 += rpp) {
+        const int r = r0 + threadIdx.x / kTPR, sub = threadIdx.x % kTPR;
+        const bool act = r < nrows;
+        T s = T(0);
+        if (act) {
+            const int i = i0 + r, c = cnt[i];
+            const size_t w = list_index(sub, i, n) / 4;
+            const uint2 *pw = (const uint2 *)nbr + w;
+            using T4 = typename V4<T>::type;
+            const T4 *pf = (const T4 *)pair_f + w;
+#pragma unroll 4
+            for (int k = sub; k < c; k += kListStripe, pw += wstep, pf += wstep) {
+                const uint2 ew = __ldcs(pw);
+                const T4 f = *pf;
+                const int e0 = (int)(ew.x & 0xffffu), e1 = (int)(ew.x >> 16), e2 = (int)(ew.y & 0xffffu),
+                          e3 = (int)(ew.y >> 16);
+                if (!QEQ_IN_BOUNDS(e0 <= total && e1 <= total && e2 <= total && e3 <= total, flags,
+                                   kSiteReal32Entry))
+                    continue;
+                s = fma(tq[e0], f.x, s);
+                s = fma(tq[e1], f.y, s);
+                s = fma(tq[e2], f.z, s);
+                s = fma(tq[e3], f.w, s);
+            }
+        }
+#pragma unroll
+        for (int o = 1; o < kTPR; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (act && sub == 0) v[(size_t)(i0 + r) * vstride] = scale * s;
     }
 }
 
@@ -1770,7 +1854,8 @@ int pme_mesh_potential(qeq_ctx *ctx, double *energy4, cudaStream_t sp) {
 
 template <typename T>
 int apply_t(qeq_ctx *ctx, const double *R, const double *q, const double *sigma, double *v,
-            double *E, double *F, double *energy4, bool need_field, bool q_only, cudaStream_t s) {
+            double *E, double *F, double *energy4, bool need_field, bool q_only, bool keep_pairs,
+            cudaStream_t s) {
     const int n = (int)ctx->n;
     using T4 = typename V4<T>::type;
     constexpr bool f64 = std::is_same<T, double>::value;
@@ -1792,7 +1877,7 @@ int apply_t(qeq_ctx *ctx, const double *R, const double *q, const double *sigma,
     prof_begin(ctx, kPhGatherIn, s);
     if (q_only) {
         k_gather_q<T><<<grid_for(n), kThreads, 0, s>>>(n, ctx->perm, q, xq, (T4 *)ctx->sfrac, fx,
-                                                       ctx->d_flags);
+                                                       (T *)ctx->q_s, ctx->d_flags);
     } else {
         int32_t *smax_bits =
             (f64 ? fl64.on : kRealLazySigma) ? ctx->d_flags + kFlagSigmaMax : nullptr;
@@ -1800,7 +1885,7 @@ int apply_t(qeq_ctx *ctx, const double *R, const double *q, const double *sigma,
         k_gather_in<T><<<grid_for(n), kThreads, 0, s>>>(
             n, ctx->perm, R, ctx->wrap_off, q, sigma, ctx->K[0] / p.box[0], ctx->K[1] / p.box[1],
             ctx->K[2] / p.box[2], xq, sg, ctx->sbase, (T4 *)ctx->sfrac, smax_bits,
-            f64 && !fl64.on ? ctx->xf_pre : nullptr, fx, ctx->d_flags);
+            f64 && !fl64.on ? ctx->xf_pre : nullptr, fx, (T *)ctx->q_s, ctx->d_flags);
         ctx->gathered = true;
     }
     prof_end(ctx, s);
@@ -1855,7 +1940,17 @@ int apply_t(qeq_ctx *ctx, const double *R, const double *q, const double *sigma,
         const dim3 grid((unsigned)ctx->geom.nbricks);
         int32_t *fl = ctx->d_flags;
         unsigned char *gt = ctx->tile_scratch;
-        if (f64 && fl64.on) {
+        const bool pair_fits = ctx->pair_f && sizeof(T) * (size_t)L.cap <= kPairSmemMax;
+        const bool sum_kept = q_only && !need_field && ctx->pair_valid && pair_fits;
+        if (!q_only) ctx->pair_valid = false;
+        const bool keep = keep_pairs && !q_only && pair_fits && (!f64 || fl64.on);
+        if (keep) ctx->pair_valid = true;
+        if (sum_kept) {
+            const T scale = f64 ? (T)std::ldexp(p.k_e, -ctx->fx_exp - kFxFBits) : (T)ra.ke_f;
+            k_pair_sum<T><<<grid, L.threads, sizeof(T) * L.cap, s>>>(
+                n, ctx->geom, ctx->tile_tab, ctx->tile_tot, ctx->nbr, ctx->cnt, (const T *)ctx->q_s,
+                (const T *)ctx->pair_f, scale, L.cap, fl, f64 ? (T *)ctx->v_s : (T *)ctx->E_s, f64 ? 1 : 4);
+        } else if (f64 && fl64.on) {
             FxArgs fa{};
             fa.nchunk = fl64.nchunk;
             fa.tpr_log2 = fl64.tpr_log2;
@@ -1873,7 +1968,8 @@ int apply_t(qeq_ctx *ctx, const double *R, const double *q, const double *sigma,
             auto launch = [&](auto kern) {
                 kern<<<fgrid, fl64.threads, fl64.smem, s>>>(
                     fa, fe, ctx->geom, ctx->tile_tab, ctx->tile_tot, ctx->nbr, ctx->cnt, ctx->xfix,
-                    ctx->sfix, pt, fl64.npair, ct, ctx->tile_cap, fl64.qcap, fl, ctx->v_s, ctx->E_s);
+                    ctx->sfix, pt, fl64.npair, ct, ctx->tile_cap, fl64.qcap, fl, ctx->v_s, ctx->E_s,
+                    keep ? (double *)ctx->pair_f : nullptr);
             };
             if (need_field && fl64.corr_smem) launch(k_real64_fixed<true, true>);
             else if (need_field) launch(k_real64_fixed<true, false>);
@@ -1896,14 +1992,19 @@ int apply_t(qeq_ctx *ctx, const double *R, const double *q, const double *sigma,
             const int32_t *sm = ctx->d_flags + kFlagSigmaMax;
             // FP32 partial sums in the E_s buffer (24 bytes per atom hold the 16)
             auto *vE32 = (float4 *)ctx->E_s;
-            if (need_field && !L.gtile)
-                k_real32<true, false><<<grid, L.threads, L.smem, s>>>(ra, ctx->geom, ctx->tile_tab, ctx->tile_tot, ctx->nbr, ctx->cnt, x4, s1, sm, L.cap, gt, fl, vE32);
-            else if (need_field)
-                k_real32<true, true><<<grid, L.threads, 0, s>>>(ra, ctx->geom, ctx->tile_tab, ctx->tile_tot, ctx->nbr, ctx->cnt, x4, s1, sm, L.cap, gt, fl, vE32);
-            else if (!L.gtile)
-                k_real32<false, false><<<grid, L.threads, L.smem, s>>>(ra, ctx->geom, ctx->tile_tab, ctx->tile_tot, ctx->nbr, ctx->cnt, x4, s1, sm, L.cap, gt, fl, vE32);
-            else
-                k_real32<false, true><<<grid, L.threads, 0, s>>>(ra, ctx->geom, ctx->tile_tab, ctx->tile_tot, ctx->nbr, ctx->cnt, x4, s1, sm, L.cap, gt, fl, vE32);
+            auto launch = [&](auto kern, size_t smem) {
+                kern<<<grid, L.threads, smem, s>>>(ra, ctx->geom, ctx->tile_tab, ctx->tile_tot, ctx->nbr, ctx->cnt,
+                                                   x4, s1, sm, L.cap, gt, fl, vE32, (float *)ctx->pair_f);
+            };
+            auto dispatch = [&](auto kept) {
+                constexpr bool K = decltype(kept)::value;
+                if (need_field && !L.gtile) launch(k_real32<true, false, K>, L.smem);
+                else if (need_field) launch(k_real32<true, true, K>, 0);
+                else if (!L.gtile) launch(k_real32<false, false, K>, L.smem);
+                else launch(k_real32<false, true, K>, 0);
+            };
+            if (keep) dispatch(std::true_type{});
+            else dispatch(std::false_type{});
         }
     }
 
@@ -2024,6 +2125,7 @@ int coulomb_alloc(qeq_ctx *ctx) {
         {(void **)&ctx->E_s, sizeof(double) * 3 * n},
         {(void **)&ctx->sbase, sizeof(int4) * n},
         {(void **)&ctx->sfrac, 4 * rs * n},
+        {&ctx->q_s, rs * n},
         {ctx->fp32 ? (void **)&ctx->xq32 : (void **)&ctx->xq64, 4 * rs * n},
         {ctx->fp32 ? (void **)&ctx->sg32 : (void **)&ctx->sg64, rs * n},
         {(void **)&ctx->xf_pre, ctx->fp32 ? 0 : sizeof(float4) * n},
@@ -2099,12 +2201,12 @@ int coulomb_alloc(qeq_ctx *ctx) {
 
     // dynamic shared memory of the tiled real-space kernels (up to 227 KB a block)
     {
-        cudaError_t ea = cudaFuncSetAttribute(k_real32<true, false>,
-                                              cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)kReal32SmemMax);
-        if (ea == cudaSuccess)
-            ea = cudaFuncSetAttribute(k_real32<false, false>,
-                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kReal32SmemMax);
+        cudaError_t ea = cudaSuccess;
+        for (const void *k : {(const void *)k_real32<true, false, false>, (const void *)k_real32<false, false, false>,
+                              (const void *)k_real32<true, false, true>, (const void *)k_real32<false, false, true>,
+                              (const void *)k_pair_sum<float>, (const void *)k_pair_sum<double>})
+            if (ea == cudaSuccess)
+                ea = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kReal32SmemMax);
         if (ea == cudaSuccess)
             ea = cudaFuncSetAttribute(k_real64<true, false>,
                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kReal64SmemMax);
@@ -2271,7 +2373,7 @@ void coulomb_free(qeq_ctx *ctx) {
     void *ptrs[] = {ctx->v_s,  ctx->E_s,  ctx->sbase, ctx->sfrac, ctx->xq32, ctx->xq64,
                     ctx->sg32, ctx->sg64, ctx->mesh,  ctx->meshc, ctx->G,    ctx->part,
                     ctx->scal, ctx->energy4, ctx->fft_work, ctx->erfc_tab64, ctx->fg_tab64, ctx->gc_tab64, ctx->xf_pre, ctx->tile_scratch,
-                    ctx->xfix, ctx->sfix, ctx->fx_tab,
+                    ctx->xfix, ctx->sfix, ctx->fx_tab, ctx->q_s, ctx->pair_f,
                     ctx->ticket};
     for (void *p : ptrs) dev_free(ctx, p);
     if (ctx->pme_stream) side_release(ctx->device, ctx->pme_stream, ctx->pme_fork, ctx->pme_join);
@@ -2354,11 +2456,46 @@ int pair64_selftest(qeq_ctx *ctx, int which, const double *arg, double *F, doubl
 
 int coulomb_apply_impl(qeq_ctx *ctx, const double *R, const double *q, const double *sigma,
                        double *v, double *E, double *F, double *energy4, bool need_field,
-                       cudaStream_t s, bool same_R) {
+                       cudaStream_t s, bool same_R, bool keep_pairs) {
     if (!ctx->list_valid) return set_error(ctx, QEQ_ERR_NOLIST, "coulomb_apply before neighbor_build");
     const bool q_only = same_R && ctx->gathered;
-    if (ctx->fp32) return apply_t<float>(ctx, R, q, sigma, v, E, F, energy4, need_field, q_only, s);
-    return apply_t<double>(ctx, R, q, sigma, v, E, F, energy4, need_field, q_only, s);
+    if (ctx->fp32)
+        return apply_t<float>(ctx, R, q, sigma, v, E, F, energy4, need_field, q_only, keep_pairs, s);
+    return apply_t<double>(ctx, R, q, sigma, v, E, F, energy4, need_field, q_only, keep_pairs, s);
+}
+
+void pair_release(qeq_ctx *ctx) {
+    dev_free(ctx, ctx->pair_f);
+    ctx->pair_f = nullptr;
+    ctx->pair_bytes = 0;
+    ctx->pair_refused = false;
+    ctx->pair_valid = false;
+}
+
+void pair_reserve(qeq_ctx *ctx, cudaStream_t s) {
+    if (ctx->pair_f || ctx->pair_refused) return;
+    // stream-ordered memory is safe on the stream it is allocated on
+    if (ctx->async_alloc && s != ctx->alloc_stream) return;
+    const size_t el = ctx->fp32 ? sizeof(float) : sizeof(double);
+    const size_t bytes = el * (size_t)ctx->width * ctx->n;
+    // the tile's charges must fit a block, and values beyond a small system's a
+    // quarter of the memory that is free (else the pairs are computed again)
+    size_t free_b = 0, total_b = 0;
+    ctx->pair_refused = true;
+    if ((!ctx->fp32 && !ctx->fx_on) || el * (size_t)ctx->tile_cap > kPairSmemMax) return;
+    if (bytes > (size_t)256 << 20 &&
+        (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess || bytes > free_b / 4)) {
+        cudaGetLastError();
+        return;
+    }
+    const std::string err = ctx->err;
+    if (dev_alloc(ctx, &ctx->pair_f, bytes) != QEQ_OK) {
+        ctx->pair_f = nullptr;
+        ctx->err = err;
+        return;
+    }
+    ctx->pair_bytes = bytes;
+    ctx->pair_refused = false;
 }
 
 }  // namespace qeq

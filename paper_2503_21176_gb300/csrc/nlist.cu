@@ -950,6 +950,7 @@ int nl_alloc_list(qeq_ctx *ctx, int width) {
                          width, kMaxWidthLimit);
     dev_free(ctx, ctx->nbr);
     dev_free(ctx, ctx->nbr_scratch);
+    pair_release(ctx);  // sized by the width
     ctx->nbr = nullptr;
     ctx->nbr_scratch = nullptr;
     int rc = dev_alloc(ctx, (void **)&ctx->nbr, sizeof(uint16_t) * (size_t)width * ctx->n);
@@ -1072,6 +1073,7 @@ static int launch_emit(qeq_ctx *ctx, cudaStream_t s) {
 int nl_build(qeq_ctx *ctx, const double *R, cudaStream_t s) {
     const int n = (int)ctx->n;
     ctx->gathered = false;  // the sorted order changes
+    ctx->pair_valid = false;
     prof_begin(ctx, kPhNeighbor, s);
     ctx->launches += 4;
     cudaMemsetAsync(ctx->cell_count, 0, sizeof(int32_t) * ctx->ncell, s);

@@ -42,9 +42,9 @@ struct FxExact {
 // A pair the fixed-point path does not decide (at the cutoff to within 2^-21, or
 // nearer than the pair table reaches; with corr_only, the Gaussian correction of a
 // pair its table does not reach, or of a very wide charge): the arithmetic of
-// k_real64, with the sorted FP64 inputs.  Adds q_j f and q_j gc d.
+// k_real64, with the sorted FP64 inputs.  Adds q_j f and q_j gc d; returns f.
 template <bool FIELD>
-__device__ __noinline__ void fx_exact_pair(const FxExact &X, int i, int j, int code, bool corr_only,
+__device__ __noinline__ double fx_exact_pair(const FxExact &X, int i, int j, int code, bool corr_only,
                                            double *acc) {
     const double4_32a xi = X.xq[i];
     double4_32a xj = X.xq[j];
@@ -55,7 +55,7 @@ __device__ __noinline__ void fx_exact_pair(const FxExact &X, int i, int j, int c
     const double dy = xj.y - xi.y;
     const double dz = xj.z - xi.z;
     const double r2 = dx * dx + dy * dy + dz * dz;
-    if (!(r2 < X.a.rc2)) return;
+    if (!(r2 < X.a.rc2)) return 0.0;
     double f = 0.0, gc = 0.0;
     if (!corr_only &&
         !pw_eval<kFGShape.oct_lo, kFGShape.sub_log2, kFGShape.ncoef>(
@@ -80,6 +80,7 @@ __device__ __noinline__ void fx_exact_pair(const FxExact &X, int i, int j, int c
         acc[2] += gq * dy;
         acc[3] += gq * dz;
     }
+    return f;
 }
 
 // Bytes of a tile atom: coordinates, charge (high word and fx_low), sigma^2.
@@ -121,7 +122,8 @@ k_real64_fixed(const __grid_constant__ FxArgs p, const __grid_constant__ FxExact
                const int32_t *__restrict__ cnt, const ulonglong4_32a *__restrict__ xfix,
                const u64 *__restrict__ sfix, const FxRow *__restrict__ pair_tab, int npair,
                const FxRow *__restrict__ corr_tab, int cap, int qcap,
-               int32_t *__restrict__ flags, double *__restrict__ v_s, double *__restrict__ E_s) {
+               int32_t *__restrict__ flags, double *__restrict__ v_s, double *__restrict__ E_s,
+               double *__restrict__ pair_f) {
     extern __shared__ __align__(32) unsigned char smem_raw[];
     __shared__ int t_start[kMaxTileBricks], t_base[kMaxTileBricks], t_code[kMaxTileBricks], t_total;
     // shared memory: pair table (npair rows), correction table, tile
@@ -130,7 +132,7 @@ k_real64_fixed(const __grid_constant__ FxArgs p, const __grid_constant__ FxExact
     ulonglong2 *tA = (ulonglong2 *)(CORR_SMEM ? ct + kFxCorrRows : ct);  // (X, Y)
     ulonglong2 *tB = tA + cap;                                                // (Z, q)
     u64 *tS = (u64 *)(tB + cap);                                              // sigma^2
-    uint16_t *cq = (uint16_t *)(tS + cap);  // the rows' queues of corrections, qcap entries a lane
+    u32 *cq = (u32 *)(tS + cap);  // the rows' queues of corrections, qcap entries a lane
     {
         const uint4 *src = (const uint4 *)pair_tab;
         uint4 *dst = (uint4 *)pt;
@@ -155,7 +157,7 @@ k_real64_fixed(const __grid_constant__ FxArgs p, const __grid_constant__ FxExact
     const unsigned row_mask = (tpr == 32 ? 0xffffffffu : (1u << tpr) - 1u) << (lane & ~(tpr - 1));
     const unsigned lt = (1u << lane) - 1u;
     // the row's queue: the entries that need the correction, in the order found
-    uint16_t *rq = cq + (size_t)(threadIdx.x >> p.tpr_log2) * qcap * tpr;
+    u32 *rq = cq + (size_t)(threadIdx.x >> p.tpr_log2) * qcap * tpr;
     const int qfull = (qcap - 4) * tpr;  // room for one more word of every lane
     // a block keeps the tables and takes every gridDim-th unit
     for (int64_t unit = blockIdx.x; unit < g.nbricks * p.nchunk; unit += gridDim.x) {
@@ -207,11 +209,18 @@ k_real64_fixed(const __grid_constant__ FxArgs p, const __grid_constant__ FxExact
         const u32 gmax = fx_hi(s2i) + smax_hi + 1;
         const u32 bound = gmax + (gmax >> 3);
         const int c = act ? cnt[i] : 0;
+        // returns the pair value it added, in units of F
         auto to_exact = [&](int e, bool corr_only) {
             if (!exact) xacc[0] = xacc[1] = xacc[2] = xacc[3] = 0.0;
             exact = true;
             const int rb = tile_locate(e, g.T, t_start, t_base);
-            fx_exact_pair<FIELD>(X, i, e - t_base[rb], t_code[rb], corr_only, xacc);
+            return scalbn(fx_exact_pair<FIELD>(X, i, e - t_base[rb], t_code[rb], corr_only, xacc),
+                          kFxFBits + p.fx_exp);
+        };
+        // kept pair values (pair_f): slot within the row's stripes as in the list
+        double *row_f = pair_f ? pair_f + (size_t)i * kListStripe : nullptr;
+        auto kept = [&](int pos) {
+            return row_f + (size_t)(pos / kListStripe) * kListStripe * X.a.n + pos % kListStripe;
         };
         // the pair's terms from F, G 2^-b and the differences
         auto add = [&](s64 F, s64 G, u64 q, s64 dx, s64 dy, s64 dz, int lz) {
@@ -277,6 +286,9 @@ k_real64_fixed(const __grid_constant__ FxArgs p, const __grid_constant__ FxExact
                 w0 = __funnelshift_r(w0, w1, 16);
                 w1 >>= 16;
                 bool queue = false;
+                // the entry's place in the row (stripe, lane's word, entry)
+                const int pos = (k0 & ~(kListStripe - 1)) + sub * 4 + u;
+                double kf = 0.0;
                 // past the row's end (padding entries are e = total)
                 if (k0 + kListLanes * u < c && e < total) {
                     const ulonglong2 aj = tA[e];
@@ -291,24 +303,27 @@ k_real64_fixed(const __grid_constant__ FxArgs p, const __grid_constant__ FxExact
                             u64 F, G = 0;
                             fx_eval<FIELD, kFxGShift>(pt[fx_piece(sh, lz)], fx_hi(y), fx_lo(y), F, G);
                             add((s64)F, (s64)G, bj.y, dx, dy, dz, lz);
+                            if (row_f) kf = (double)F;
                             if ((sh >> 3) < bound) {
                                 const u32 gh = fx_hi(s2i + tS[e]);
                                 queue = (sh >> 3) < gh + (gh >> 3);
                             }
                         } else {
-                            to_exact(e, false);
+                            kf = to_exact(e, false);
                         }
                     }
                 }
+                if (row_f && k0 < c) *kept(pos) = kf;
                 const unsigned m = __ballot_sync(0xffffffffu, queue) & row_mask;
-                if (queue) rq[nq + __popc(m & lt)] = (uint16_t)e;
+                if (queue) rq[nq + __popc(m & lt)] = (u32)e | (u32)pos << 16;
                 nq += __popc(m);
             }
             fold();
             if (left > 0 && !__any_sync(0xffffffffu, nq > qfull)) continue;
             __syncwarp();
             for (int m = l; m < nq; m += tpr) {
-                const int e = rq[m];
+                const u32 qe = rq[m];
+                const int e = (int)(qe & 0xffffu);
                 const ulonglong2 aj = tA[e];
                 const ulonglong2 bj = tB[e];
                 const s64 dx = (s64)(aj.x - ai.x), dy = (s64)(aj.y - ai.y), dz = (s64)(bj.x - zi);
@@ -319,8 +334,10 @@ k_real64_fixed(const __grid_constant__ FxArgs p, const __grid_constant__ FxExact
                 if (g2 < kFxSigmaSat && fx_correct<FIELD>(corr, s, fx_bshift(lz), g2, F, G)) {
                     add(F, G, bj.y, dx, dy, dz, lz);
                     fold();
+                    if (row_f) *kept((int)(qe >> 16)) += (double)F;
                 } else {
-                    to_exact(e, true);
+                    const double kf = to_exact(e, true);
+                    if (row_f) *kept((int)(qe >> 16)) += kf;
                 }
             }
             nq = 0;
@@ -403,7 +420,7 @@ inline FxLaunch fx_launch(const qeq_ctx *ctx) {
     // shared memory: the pair table, the tile and the shortest queues must fit; the
     // correction table comes in where it leaves room for them, the queues take up
     // to kFxQueue entries of the rest
-    const size_t slot = sizeof(uint16_t) * L.threads;
+    const size_t slot = sizeof(u32) * L.threads;
     const size_t base = sizeof(FxRow) * L.npair + (size_t)ctx->tile_cap * kFxTileBytes;
     if (base + 4 * slot > kReal64SmemMax) return L;
     L.corr_smem = base + kFxCorrBytes + 4 * slot <= kReal64SmemMax;

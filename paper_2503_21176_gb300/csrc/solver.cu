@@ -241,7 +241,7 @@ int plain_apply(qeq_ctx *ctx, const double *R, const double *u, const double *si
                 const double *x, double *y, cudaStream_t s, bool same_R) {
     const int n = (int)ctx->n;
     int rc = coulomb_apply_impl(ctx, R, x, sigma, ctx->phi, nullptr, nullptr, nullptr, false, s,
-                                same_R);
+                                same_R, true);
     if (rc) return rc;
     k_bordered_apply<<<ctx->red_grid, kThreads, 0, s>>>(n, u, ctx->phi, x, y, ctx->part);
     launch_finalize(ctx, ctx->part, 1, ctx->gmH + 2 * (kMaxDots + 2) + 1, s);
@@ -273,6 +273,7 @@ int gmres_solve(qeq_ctx *ctx, const double *R, const double *chi, const double *
     restart = std::max(1, std::min(restart, kMaxDots));
     int rc = solver_alloc(ctx, restart);
     if (rc) return rc;
+    pair_reserve(ctx, s);  // every iteration's apply is at these positions
     const qeq_params &p = ctx->p;
     k_jacobi<<<ctx->red_grid, kThreads, 0, s>>>(n, u, sigma, p.gaussian_self ? p.k_e * kSqrtTwoOverPi : 0.0,
                                              ctx->gmDinv);

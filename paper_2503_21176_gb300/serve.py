@@ -103,7 +103,8 @@ def estimate_device_bytes(req: Request) -> int:
     K0, K1, K2 = req.mesh
     mesh = K0 * K1 * K2
     meshc = K0 * K1 * (K2 // 2 + 1)
-    per_atom = 4 * width + 8 * (3 * 12 + 2 * req.rank + req.k_d + 16) + 16 * rs + 64
+    # list, emit scratch and kept pair values; the fixed-point inputs of FP64
+    per_atom = (6 + rs) * width + (40 if rs == 8 else 0) + 8 * (3 * 12 + 2 * req.rank + req.k_d + 16) + 16 * rs + 64
     total = n * per_atom + rs * (mesh + 3 * 2 * meshc + 2 * mesh)
     return int(1.25 * total) + (4 << 20)
 
