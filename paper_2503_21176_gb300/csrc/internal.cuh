@@ -141,10 +141,12 @@ __host__ __device__ __forceinline__ int64_t brick_index(const BrickGeom &g, int 
     return ((int64_t)bx * g.nb[1] + by) * g.nb[2] + bz;
 }
 
-// Brick-major index of cell (cx, cy, cz), 0 <= c < nc.
+// Brick-major index of cell (cx, cy, cz), 0 <= c < nc.  Bricks are 1 or 2 cells per
+// axis, so division by B is a shift by B - 1.
 __host__ __device__ __forceinline__ int cell_index(const BrickGeom &g, int cx, int cy, int cz) {
-    const int bx = cx / g.B[0], by = cy / g.B[1], bz = cz / g.B[2];
-    const int lx = cx - bx * g.B[0], ly = cy - by * g.B[1], lz = cz - bz * g.B[2];
+    const int mx = g.B[0] - 1, my = g.B[1] - 1, mz = g.B[2] - 1;
+    const int bx = cx >> mx, by = cy >> my, bz = cz >> mz;
+    const int lx = cx & mx, ly = cy & my, lz = cz & mz;
     return (int)(brick_index(g, bx, by, bz) * g.bvol + (lx * g.B[1] + ly) * g.B[2] + lz);
 }
 

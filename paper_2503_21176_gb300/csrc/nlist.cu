@@ -29,16 +29,42 @@ namespace qeq {
 
 namespace {
 
-__global__ void k_wrap_bin(int n, const double *__restrict__ R, double Lx, double Ly, double Lz,
-                           double cwx, double cwy, double cwz, BrickGeom g,
-                           int32_t *__restrict__ cell_of, int32_t *__restrict__ cell_count,
+// x / L rounded down, as floor of the IEEE quotient: from x times 1 / L where that is
+// more than 2^-20 away from a whole number (its error is below 2^-31 for |x / L| <
+// 2^20), else by the division, on GB300's 1/64-rate FP64 pipe some 20 times the work
+// (k_wrap_bin at 300,000 atoms: 41.6 us with two divisions a coordinate, 24.7 us so).
+__device__ __forceinline__ double floor_quotient(double x, double L, double inv_L) {
+    const double t = x * inv_L;
+    const double fl = floor(t);
+    const int hf = __double2hiint(t - fl);  // of the fraction in [0, 1)
+    const int ht = __double2hiint(t) & 0x7fffffff;
+    if (hf > 0x3EB00000 && hf < 0x3FEFFFFE && ht < 0x41300000) return fl;
+    return floor(__ddiv_rn(x, L));
+}
+
+// Box edges and cell widths, with their reciprocals from the host.
+struct WrapArgs {
+    double L[3], cw[3], inv_L[3], inv_cw[3];
+};
+
+WrapArgs wrap_args(const double *L, const double *cw) {
+    WrapArgs w;
+    for (int d = 0; d < 3; ++d) {
+        w.L[d] = L[d];
+        w.cw[d] = cw[d];
+        w.inv_L[d] = 1.0 / L[d];
+        w.inv_cw[d] = 1.0 / cw[d];
+    }
+    return w;
+}
+
+__global__ void k_wrap_bin(int n, const double *__restrict__ R, const __grid_constant__ WrapArgs a,
+                           const __grid_constant__ BrickGeom g, int32_t *__restrict__ cell_of,
+                           int32_t *__restrict__ cell_count,
                            double *__restrict__ wrap_off, double *__restrict__ R_build,
                            int32_t *__restrict__ flags) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    const double L[3] = {Lx, Ly, Lz};
-    const double cw[3] = {cwx, cwy, cwz};
-    const int nc[3] = {g.nc[0], g.nc[1], g.nc[2]};
     int c[3];
     bool finite = true;
 #pragma unroll
@@ -46,13 +72,13 @@ __global__ void k_wrap_bin(int n, const double *__restrict__ R, double Lx, doubl
         const double x = R[3 * (size_t)i + d];
         finite = finite && isfinite(x);
         // w = -(L * floor(x / L)), xw = x + w: one IEEE rounding per operation
-        const double fl = floor(__ddiv_rn(x, L[d]));
-        const double w = -__dmul_rn(L[d], fl);
+        const double fl = floor_quotient(x, a.L[d], a.inv_L[d]);
+        const double w = -__dmul_rn(a.L[d], fl);
         const double xw = __dadd_rn(x, w);
         wrap_off[3 * (size_t)i + d] = w;
         R_build[3 * (size_t)i + d] = x;
-        int cc = isfinite(xw) ? (int)floor(xw / cw[d]) : 0;
-        c[d] = min(max(cc, 0), nc[d] - 1);
+        const int cc = isfinite(xw) ? (int)floor_quotient(xw, a.cw[d], a.inv_cw[d]) : 0;
+        c[d] = min(max(cc, 0), g.nc[d] - 1);
     }
     if (!finite) atomicExch(&flags[kFlagNonFinite], 1);
     const int cell = cell_index(g, c[0], c[1], c[2]);
@@ -1079,8 +1105,8 @@ int nl_build(qeq_ctx *ctx, const double *R, cudaStream_t s) {
     cudaMemsetAsync(ctx->cell_count, 0, sizeof(int32_t) * ctx->ncell, s);
     cudaMemsetAsync(ctx->d_flags, 0, sizeof(int32_t) * kFlagBounds, s);  // the bounds flag persists
     k_wrap_bin<<<grid_for(n), kThreads, 0, s>>>(
-        n, R, ctx->p.box[0], ctx->p.box[1], ctx->p.box[2], ctx->cw[0], ctx->cw[1], ctx->cw[2],
-        ctx->geom, ctx->cell_of, ctx->cell_count, ctx->wrap_off, ctx->R_build, ctx->d_flags);
+        n, R, wrap_args(ctx->p.box, ctx->cw), ctx->geom, ctx->cell_of, ctx->cell_count,
+        ctx->wrap_off, ctx->R_build, ctx->d_flags);
     k_scan<<<1, kScanThreads, 0, s>>>(ctx->ncell, ctx->cell_count, ctx->cell_start, ctx->cell_fill);
     k_scatter<<<grid_for(n), kThreads, 0, s>>>(n, ctx->cell_of, ctx->cell_start, ctx->cell_fill,
                                                ctx->tmp_list);
@@ -1432,9 +1458,8 @@ QEQ_API int qeq_neighbor_build_noalloc(const double *R, int64_t n_atoms, const d
         g.B[d] = 1;
     }
     g.bvol = 1;
-    k_wrap_bin<<<grid_for(n), kThreads, 0, s>>>(n, R, box[0], box[1], box[2], cw[0], cw[1], cw[2],
-                                                g, S->cell_of, S->cell_count, S->wrap_off,
-                                                S->R_build, S->flags);
+    k_wrap_bin<<<grid_for(n), kThreads, 0, s>>>(n, R, wrap_args(box, cw), g, S->cell_of,
+                                                S->cell_count, S->wrap_off, S->R_build, S->flags);
     k_scan<<<1, kScanThreads, 0, s>>>(ncell, S->cell_count, S->cell_start, S->cell_fill);
     k_scatter<<<grid_for(n), kThreads, 0, s>>>(n, S->cell_of, S->cell_start, S->cell_fill,
                                                S->tmp_list);
