@@ -10,7 +10,9 @@
 // ||b - A z|| / ||b||.  That is the paper's tolerance.  Each Arnoldi vector
 // costs one potential-only Coulomb apply.  Vectors have N + 1 entries, the
 // last one being lambda.  Orthogonalisation is classical Gram-Schmidt done
-// twice, each pass one multi-dot kernel plus one update kernel.  The
+// twice in three kernels; an iteration is five launches beside its apply (sums
+// finish in the last block of their kernel, scaling runs with the preconditioner,
+// a subtraction with the dots or the norm that follow it).  The
 // (m + 1) x m Hessenberg least-squares problem is reduced by Givens rotations
 // on the host from one small device-to-host copy per iteration.
 //
@@ -31,10 +33,10 @@ namespace {
 constexpr int kMaxDots = kMaxGmresRestart;  // Gram-Schmidt against at most this many vectors
 
 // y = A x for x = [xq; xl]:  y_q = u o xq + Phi xq + xl,  y_l = sum xq.
-// phi holds Phi xq.  The partial of sum xq goes to part slot 0.
+// phi holds Phi xq; the last block to finish writes y_l.
 __global__ void k_bordered_apply(int n, const double *__restrict__ u, const double *__restrict__ phi,
                                  const double *__restrict__ x, double *__restrict__ y,
-                                 double *__restrict__ part) {
+                                 double *__restrict__ part, unsigned int *__restrict__ ticket) {
     const double xl = x[n];
     double s = 0.0;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
@@ -44,55 +46,106 @@ __global__ void k_bordered_apply(int n, const double *__restrict__ u, const doub
     double vals[1] = {s};
     block_sum<1>(vals);
     if (threadIdx.x == 0) part[blockIdx.x] = vals[0];
+    finalize_last_block<1>(part, y + n, ticket);
 }
 
-// last entry of y from the finalized sum
-__global__ void k_set_last(int n, const double *__restrict__ src, double *__restrict__ y) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) y[n] = src[0];
-}
-
-// z = M^{-1} x (q part divided by d, lambda unchanged)
-__global__ void k_precond(int n, const double *__restrict__ dinv, const double *__restrict__ x,
-                          double *__restrict__ z) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i <= n; i += gridDim.x * blockDim.x)
-        z[i] = i < n ? x[i] * dinv[i] : x[i];
-}
-
-// partials of <V_k, w> for k < nv over n + 1 entries (slot k), and of <w, w> (slot nv)
-__global__ void k_multi_dot(int n1, int nv, const double *__restrict__ V, const double *__restrict__ w,
-                            double *__restrict__ part) {
-    for (int k = 0; k <= nv; ++k) {
-        const double *a = k < nv ? V + (size_t)k * n1 : w;
-        double s = 0.0;
-        for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n1; i += gridDim.x * blockDim.x)
-            s += a[i] * w[i];
-        double vals[1] = {s};
-        block_sum<1>(vals);
-        if (threadIdx.x == 0) part[(size_t)k * kRedBlocks + blockIdx.x] = vals[0];
+// v = a x over n + 1 entries, and z = M^{-1} v (q part times dinv, lambda unchanged);
+// v may be x.
+__global__ void k_scale_precond(int n, double a, const double *x, double *v,
+                                const double *__restrict__ dinv, double *__restrict__ z) {
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i <= n; i += gridDim.x * blockDim.x) {
+        const double t = a * x[i];
+        v[i] = t;
+        z[i] = i < n ? t * dinv[i] : t;
     }
 }
 
-// w -= sum_k h_k V_k
-__global__ void k_subtract(int n1, int nv, const double *__restrict__ V, const double *__restrict__ h,
-                           double *__restrict__ w) {
+// Partials of <V_k, w>, k < nv, over n1 entries (slot k): eight vectors a pass, so w is
+// read once for them and their sums fold together.
+__device__ __forceinline__ void dots(int n1, int nv, const double *__restrict__ V, const double *w,
+                                     double *__restrict__ part) {
+    for (int k0 = 0; k0 < nv; k0 += 8) {
+        double s[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+        for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n1; i += gridDim.x * blockDim.x) {
+            const double wi = w[i];
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+                if (k0 + u < nv) s[u] = fma(V[(size_t)(k0 + u) * n1 + i], wi, s[u]);
+        }
+        block_sum<8>(s);
+        if (threadIdx.x == 0)
+            for (int u = 0; u < 8 && k0 + u < nv; ++u) part[(size_t)(k0 + u) * kRedBlocks + blockIdx.x] = s[u];
+    }
+}
+
+// The last block to arrive sums nslots slots' partials in a fixed order, one warp a slot.
+__device__ __forceinline__ void finalize_slots(int nslots, const double *part, double *out,
+                                               unsigned int *ticket) {
+    __shared__ bool is_last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) is_last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!is_last) return;
+    __threadfence();
+    const int lane = threadIdx.x & 31;
+    for (int k = threadIdx.x >> 5; k < nslots; k += kThreads / 32) {
+        double t = 0.0;
+        for (int b = lane; b < (int)gridDim.x; b += 32) t += __ldcg(part + (size_t)k * kRedBlocks + b);
+        t = warp_sum(t);
+        if (lane == 0) out[k] = t;
+    }
+    if (threadIdx.x == 0) *ticket = 0u;
+}
+
+// h_k = <V_k, w>, k < nv
+__global__ void k_multi_dot(int n1, int nv, const double *__restrict__ V, const double *__restrict__ w,
+                            double *__restrict__ part, double *__restrict__ h,
+                            unsigned int *__restrict__ ticket) {
+    dots(n1, nv, V, w, part);
+    finalize_slots(nv, part, h, ticket);
+}
+
+// w -= sum_k h_k V_k, then (again) h2_k = <V_k, w> or (norm) h2_0 = <w, w>: each thread
+// owns its entries of w, so the subtraction and the next dots need one launch.
+__global__ void k_subtract_dot(int n1, int nv, const double *__restrict__ V, const double *__restrict__ h,
+                               double *w, bool norm, double *__restrict__ part, double *__restrict__ h2,
+                               unsigned int *__restrict__ ticket) {
+    __shared__ double hs[kMaxDots];
+    for (int k = threadIdx.x; k < nv; k += blockDim.x) hs[k] = h[k];
+    __syncthreads();
+    double n2 = 0.0;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n1; i += gridDim.x * blockDim.x) {
         double s = w[i];
-        for (int k = 0; k < nv; ++k) s -= h[k] * V[(size_t)k * n1 + i];
+        for (int k = 0; k < nv; ++k) s -= hs[k] * V[(size_t)k * n1 + i];
         w[i] = s;
+        n2 = fma(s, s, n2);
+    }
+    if (norm) {
+        double vals[1] = {n2};
+        block_sum<1>(vals);
+        if (threadIdx.x == 0) part[blockIdx.x] = vals[0];
+        finalize_last_block<1>(part, h2, ticket);
+    } else {
+        dots(n1, nv, V, w, part);
+        finalize_slots(nv, part, h2, ticket);
     }
 }
 
-// y = a * x   (n1 entries)
-__global__ void k_scale(int n1, double a, const double *__restrict__ x, double *__restrict__ y) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n1; i += gridDim.x * blockDim.x)
-        y[i] = a * x[i];
-}
-
-// r = b - Az with b = [-chi; q_tot]
-__global__ void k_residual(int n, double q_tot, const double *__restrict__ chi,
-                           const double *__restrict__ Az, double *__restrict__ r) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i <= n; i += gridDim.x * blockDim.x)
-        r[i] = (i < n ? -chi[i] : q_tot) - Az[i];
+// r = b - Az with b = [-chi; q_tot] (Az null: b itself), and |r|^2; r may be Az
+__global__ void k_residual(int n, double q_tot, const double *__restrict__ chi, const double *Az, double *r,
+                           double *__restrict__ part, double *__restrict__ r2,
+                           unsigned int *__restrict__ ticket) {
+    double s = 0.0;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i <= n; i += gridDim.x * blockDim.x) {
+        const double ri = (i < n ? -chi[i] : q_tot) - (Az ? Az[i] : 0.0);
+        r[i] = ri;
+        s = fma(ri, ri, s);
+    }
+    double vals[1] = {s};
+    block_sum<1>(vals);
+    if (threadIdx.x == 0) part[blockIdx.x] = vals[0];
+    finalize_last_block<1>(part, r2, ticket);
 }
 
 // z += M^{-1} (sum_k y_k V_k)
@@ -191,25 +244,24 @@ void solver_free(qeq_ctx *ctx) {
 
 namespace {
 
-// Orthogonalise w against V_0..V_{nv-1}, classical Gram-Schmidt twice.
+// Orthogonalise w against V_0..V_{nv-1}, classical Gram-Schmidt twice: three launches
+// (dots; subtract and dots again; subtract and norm).  Small vectors are bound by the
+// launches: 20,000 atoms in FP64 took 17.3 ms with twelve launches an iteration beside
+// the apply, 14.2 ms with five.  Long ones are bound by reading V four times.
 // On return h[k] is the sum of both passes' coefficients and norm = |w|.
 int cgs2(qeq_ctx *ctx, int n1, int nv, double *w, std::vector<double> &h, double &norm,
          cudaStream_t s) {
     double *part = ctx->part;
     double *dh = ctx->gmH;  // pass 1 at [0, nv), pass 2 at [kMaxDots + 2, ...), |w|^2 at the end
     const int off2 = kMaxDots + 2;
-    for (int pass = 0; pass < 2; ++pass) {
-        double *dst = dh + (pass == 0 ? 0 : off2);
-        k_multi_dot<<<ctx->red_grid, kThreads, 0, s>>>(n1, nv, ctx->gmV, w, part);
-        launch_finalize(ctx, part, nv, dst, s);
-        k_subtract<<<ctx->red_grid, kThreads, 0, s>>>(n1, nv, ctx->gmV, dst, w);
-        ctx->launches += 3;
-    }
-    k_multi_dot<<<ctx->red_grid, kThreads, 0, s>>>(n1, 0, ctx->gmV, w, part);
-    launch_finalize(ctx, part, 1, dh + 2 * off2, s);
-    ctx->launches += 2;
-    std::vector<double> hb(2 * off2 + 1);
-    cudaError_t e = cudaMemcpyAsync(hb.data(), dh, sizeof(double) * hb.size(), cudaMemcpyDeviceToHost, s);
+    const int G = ctx->atom_grid;
+    k_multi_dot<<<G, kThreads, 0, s>>>(n1, nv, ctx->gmV, w, part, dh, ctx->ticket);
+    k_subtract_dot<<<G, kThreads, 0, s>>>(n1, nv, ctx->gmV, dh, w, false, part, dh + off2, ctx->ticket);
+    k_subtract_dot<<<G, kThreads, 0, s>>>(n1, nv, ctx->gmV, dh + off2, w, true, part, dh + 2 * off2,
+                                          ctx->ticket);
+    ctx->launches += 3;
+    double hb[2 * (kMaxDots + 2) + 1];
+    cudaError_t e = cudaMemcpyAsync(hb, dh, sizeof(hb), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     int rc = cuda_check(ctx, e, "gmres orthogonalise");
     if (rc) return rc;
@@ -219,41 +271,23 @@ int cgs2(qeq_ctx *ctx, int n1, int nv, double *w, std::vector<double> &h, double
     return QEQ_OK;
 }
 
-// y = A M^{-1} x  (one potential-only Coulomb apply)
-int precond_apply(qeq_ctx *ctx, const double *R, const double *u, const double *sigma,
-                  const double *x, double *y, cudaStream_t s, bool same_R) {
-    const int n = (int)ctx->n;
-    double *z = ctx->gmZ;
-    k_precond<<<ctx->red_grid, kThreads, 0, s>>>(n, ctx->gmDinv, x, z);
-    ctx->launches++;
-    int rc = coulomb_apply_impl(ctx, R, z, sigma, ctx->phi, nullptr, nullptr, nullptr, false, s,
-                                same_R);
-    if (rc) return rc;
-    k_bordered_apply<<<ctx->red_grid, kThreads, 0, s>>>(n, u, ctx->phi, z, y, ctx->part);
-    launch_finalize(ctx, ctx->part, 1, ctx->gmH + 2 * (kMaxDots + 2) + 1, s);
-    k_set_last<<<1, 32, 0, s>>>(n, ctx->gmH + 2 * (kMaxDots + 2) + 1, y);
-    ctx->launches += 3;
-    return QEQ_OK;
-}
-
-// A x without preconditioning (x in gmZ already as a plain vector)
-int plain_apply(qeq_ctx *ctx, const double *R, const double *u, const double *sigma,
-                const double *x, double *y, cudaStream_t s, bool same_R) {
+// y = A x  (one potential-only Coulomb apply)
+int bordered_apply(qeq_ctx *ctx, const double *R, const double *u, const double *sigma,
+                   const double *x, double *y, cudaStream_t s, bool same_R) {
     const int n = (int)ctx->n;
     int rc = coulomb_apply_impl(ctx, R, x, sigma, ctx->phi, nullptr, nullptr, nullptr, false, s,
                                 same_R, true);
     if (rc) return rc;
-    k_bordered_apply<<<ctx->red_grid, kThreads, 0, s>>>(n, u, ctx->phi, x, y, ctx->part);
-    launch_finalize(ctx, ctx->part, 1, ctx->gmH + 2 * (kMaxDots + 2) + 1, s);
-    k_set_last<<<1, 32, 0, s>>>(n, ctx->gmH + 2 * (kMaxDots + 2) + 1, y);
-    ctx->launches += 3;
+    k_bordered_apply<<<ctx->atom_grid, kThreads, 0, s>>>(n, u, ctx->phi, x, y, ctx->part, ctx->ticket);
+    ctx->launches++;
     return QEQ_OK;
 }
 
-double host_norm(qeq_ctx *ctx, const double *x, int n1, cudaStream_t s, int *rc) {
-    k_multi_dot<<<ctx->red_grid, kThreads, 0, s>>>(n1, 0, ctx->gmV, x, ctx->part);
-    launch_finalize(ctx, ctx->part, 1, ctx->gmH, s);
-    ctx->launches += 2;
+// r = b - Az (Az null: b) and its norm on the host
+double residual_norm(qeq_ctx *ctx, const double *chi, const double *Az, double *r, cudaStream_t s, int *rc) {
+    k_residual<<<ctx->atom_grid, kThreads, 0, s>>>((int)ctx->n, ctx->p.q_tot, chi, Az, r, ctx->part, ctx->gmH,
+                                                   ctx->ticket);
+    ctx->launches++;
     double v = 0.0;
     cudaError_t e = cudaMemcpyAsync(&v, ctx->gmH, sizeof(double), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
@@ -280,11 +314,8 @@ int gmres_solve(qeq_ctx *ctx, const double *R, const double *chi, const double *
     ctx->launches++;
     double *w = ctx->gmW;       // A z, then the residual / Arnoldi work vector
     double *bvec = ctx->gmW + n1;
-    // |b| with b = [-chi; q_tot]  (residual of A z = 0)
-    cudaMemsetAsync(w, 0, sizeof(double) * n1, s);
-    k_residual<<<ctx->red_grid, kThreads, 0, s>>>(n, p.q_tot, chi, w, bvec);
-    ctx->launches++;
-    double bnorm = host_norm(ctx, bvec, n1, s, &rc);
+    // |b| with b = [-chi; q_tot]
+    double bnorm = residual_norm(ctx, chi, nullptr, bvec, s, &rc);
     if (rc) return rc;
     if (!(bnorm > 0.0)) bnorm = 1.0;
     int iters = 0, applies = 0;
@@ -292,24 +323,24 @@ int gmres_solve(qeq_ctx *ctx, const double *R, const double *chi, const double *
     std::vector<double> H((size_t)(restart + 1) * restart), cs(restart), sn(restart), g(restart + 1), h;
     while (true) {
         // r = b - A z
-        rc = plain_apply(ctx, R, u, sigma, z, w, s, applies > 0);
+        rc = bordered_apply(ctx, R, u, sigma, z, w, s, applies > 0);
         if (rc) return rc;
         ++applies;
-        k_residual<<<ctx->red_grid, kThreads, 0, s>>>(n, p.q_tot, chi, w, w);
-        ctx->launches++;
-        const double beta = host_norm(ctx, w, n1, s, &rc);
+        const double beta = residual_norm(ctx, chi, w, w, s, &rc);
         if (rc) return rc;
         relres = beta / bnorm;
         if (relres <= tol || iters >= max_iter || !(beta > 0.0)) break;
-        k_scale<<<ctx->red_grid, kThreads, 0, s>>>(n1, 1.0 / beta, w, ctx->gmV);
-        ctx->launches++;
         std::fill(g.begin(), g.end(), 0.0);
         g[0] = beta;
+        double scale = 1.0 / beta;  // of the vector that becomes V_j, still unscaled in from
+        const double *from = w;
         int j = 0;
         for (; j < restart && iters < max_iter; ++j) {
             double *vj = ctx->gmV + (size_t)j * n1;
             double *vnext = ctx->gmV + (size_t)(j + 1) * n1;
-            rc = precond_apply(ctx, R, u, sigma, vj, vnext, s, applies > 0);
+            k_scale_precond<<<ctx->atom_grid, kThreads, 0, s>>>(n, scale, from, vj, ctx->gmDinv, ctx->gmZ);
+            ctx->launches++;
+            rc = bordered_apply(ctx, R, u, sigma, ctx->gmZ, vnext, s, applies > 0);
             if (rc) return rc;
             ++applies;
             ++iters;
@@ -318,10 +349,8 @@ int gmres_solve(qeq_ctx *ctx, const double *R, const double *chi, const double *
             if (rc) return rc;
             for (int k = 0; k <= j; ++k) H[(size_t)k * restart + j] = h[k];
             H[(size_t)(j + 1) * restart + j] = hn;
-            if (hn > 0.0) {
-                k_scale<<<ctx->red_grid, kThreads, 0, s>>>(n1, 1.0 / hn, vnext, vnext);
-                ctx->launches++;
-            }
+            scale = hn > 0.0 ? 1.0 / hn : 1.0;
+            from = vnext;
             // apply the previous rotations to column j, then a new one
             for (int k = 0; k < j; ++k) {
                 const double a = H[(size_t)k * restart + j], b = H[(size_t)(k + 1) * restart + j];
@@ -360,12 +389,10 @@ int gmres_solve(qeq_ctx *ctx, const double *R, const double *chi, const double *
         if ((relres <= tol || iters >= max_iter) && !final_check) break;
         if (relres <= tol || iters >= max_iter) {
             // true residual of the final iterate (one more apply)
-            rc = plain_apply(ctx, R, u, sigma, z, w, s, applies > 0);
+            rc = bordered_apply(ctx, R, u, sigma, z, w, s, applies > 0);
             if (rc) return rc;
             ++applies;
-            k_residual<<<ctx->red_grid, kThreads, 0, s>>>(n, p.q_tot, chi, w, w);
-            ctx->launches++;
-            relres = host_norm(ctx, w, n1, s, &rc) / bnorm;
+            relres = residual_norm(ctx, chi, w, w, s, &rc) / bnorm;
             if (rc) return rc;
             break;
         }
