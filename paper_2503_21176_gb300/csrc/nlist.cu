@@ -1076,6 +1076,9 @@ static int launch_emit(qeq_ctx *ctx, cudaStream_t s) {
         const int nchunk = (int)std::max<int64_t>(
             1, std::min<int64_t>((groups + kGroupThreads / 32 - 1) / (kGroupThreads / 32),
                                  (4 * (int64_t)ctx->sm_count + nb - 1) / nb));
+        // its class counts are nested: the near radius ends at the cutoff, which a skin
+        // above 0.73 r_cut would leave behind
+        a.t_near = std::min(a.t_near, a.t_cut);
         k_emit_group<<<(unsigned)(nb * nchunk), kGroupThreads, 0, s>>>(
             a, ctx->geom, nchunk, rpg, ctx->xs64, ctx->xs32, ctx->cell_start, ctx->nbr, ctx->cnt,
             ctx->tile_tab, ctx->tile_tot, ctx->d_flags);

@@ -26,3 +26,16 @@ def test_grouped_list_is_exact(n, box, r_list, width):
     rows = canonical_rows_gpu(*s.neighbor_export())
     assert rows == canonical_rows_oracle(*neighbors.brute_force_pairs(R, box, r_list))
     s.close()
+
+
+def test_skin_wider_than_the_near_class():
+    """r_list^2 / 3 > r_cut^2: the near radius lies beyond the cutoff."""
+    qg = cuda_or_skip()
+    rng = np.random.default_rng(5)
+    box = np.array([11.0, 12.0, 13.0])
+    R = rng.uniform(0, 1, (900, 3)) * box
+    s = qg.System(qg.make_params(900, box, r_cut=1.8, skin=1.9, mesh=(16, 16, 16)))
+    s.neighbor_build(dev_tensor(R))
+    rows = canonical_rows_gpu(*s.neighbor_export())
+    assert rows == canonical_rows_oracle(*neighbors.brute_force_pairs(R, box, 3.7))
+    s.close()
