@@ -497,8 +497,9 @@ def roofline(res, precision, n_pairs_rc, peaks, pipes):
 
     The real-space kernel is bound by the arithmetic pipes, so its fraction is the
     method's floating-point work (PAIR_FLOPS per directed pair inside r_c) over
-    the FP32 (or FP64) FMA rate measured on this GPU by qeq_measure_peaks; the
-    special-function work is quoted beside it against the measured MUFU rate."""
+    the FP32 FMA rate measured on this GPU by qeq_measure_peaks; the
+    special-function work is quoted beside it against the measured MUFU rate.
+    The FP64 context's pairs run on the integer pipes: no fraction is given."""
     prof = res.get("_profile") or {}
     if not prof:
         return None
@@ -511,7 +512,10 @@ def roofline(res, precision, n_pairs_rc, peaks, pipes):
         achieved = n_pairs_rc * PAIR_FLOPS / (avg_ms * 1e-3) / 1e12
         sfu = n_pairs_rc * PAIR_SFU / (avg_ms * 1e-3)
         out = {"kernel": name, "bound": "alu", "achieved": round(achieved, 4),
-               "peak": round(peak, 3), "unit": "TFLOP/s", "frac": round(achieved / peak, 4),
+               "peak": round(peak, 3), "unit": "TFLOP/s", "frac": round(achieved / peak, 4) if fp32 else None,
+               "note": "average over the launch of a step that computes the pairs and those that sum "
+                       "its kept pair values" + ("" if fp32 else "; the pairs are computed in 64-bit fixed "
+                       "point on the integer pipes, so the FP64 pipe's rate is no ceiling of theirs"),
                "traffic": REAL32_TRAFFIC_BYTES if fp32 else REAL64_TRAFFIC_BYTES,
                "traffic_unit": "DRAM bytes per launch (ncu, scaled from 120k atoms)",
                "algorithmic": f"{PAIR_FLOPS} flop x {n_pairs_rc} directed pairs inside r_c "
