@@ -268,8 +268,8 @@ __device__ __noinline__ bool band_keep(const EmitArgs *ap, int code, const doubl
 // classes are counted; counts keep running past cap (an overflow, reported for
 // the regrowth).
 __device__ __forceinline__ void emit_cells(const EmitArgs &a, const EmitArgs *sa, int i, int s,
-                                           const int4 *__restrict__ tab,
-                                           const float4 *__restrict__ shtab, int ncand,
+                                           const uint2 *__restrict__ tab, const int *t_base,
+                                           const int *t_code, const float4 *__restrict__ shtab, int ncand,
                                            const float4 &xf,
                                            const double4_32a *__restrict__ xs64,
                                            const float4 *__restrict__ xs32, int cap, int (&c)[3],
@@ -280,18 +280,20 @@ __device__ __forceinline__ void emit_cells(const EmitArgs &a, const EmitArgs *sa
     size_t base = (size_t)i * kListStripe + (size_t)s * 4u;
     int m = 0, near = 0, inside = 0;
     for (int k = 0; k < ncand; ++k) {
-        const int4 ct = tab[k];
-        const float4 sh = shtab[ct.w];
+        const uint2 ct = tab[k];
+        const int rb = ct.y & 127u, code = t_code[rb], tbase = t_base[rb];
+        const int end = (int)(ct.x + (ct.y >> 7));
+        const float4 sh = shtab[code];
         const float px = xf.x - sh.x, py = xf.y - sh.y, pz = xf.z - sh.z;
-        const bool home = ct.w == kCenterCode;
-        for (int j = ct.x + s; j < ct.y; j += kEmitLanes) {
+        const bool home = code == kCenterCode;
+        for (int j = (int)ct.x + s; j < end; j += kEmitLanes) {
             const float4 xj = xs32[j];
             const float dxf = xj.x - px, dyf = xj.y - py, dzf = xj.z - pz;
             const float d2f = fmaf(dzf, dzf, fmaf(dyf, dyf, dxf * dxf));
             if (d2f > a.hi) continue;
             if (home && j == i) continue;
-            if (!(d2f < a.lo) && !band_keep(sa, ct.w, xs64 + j, xs64 + i)) continue;
-            const int e = j + ct.z;
+            if (!(d2f < a.lo) && !band_keep(sa, code, xs64 + j, xs64 + i)) continue;
+            const int e = j + tbase;
             if (!QEQ_IN_BOUNDS((unsigned)e < (unsigned)t_total, flags, kSiteEmitTile)) continue;
             const int cls = (d2f >= a.t_near) + (d2f >= a.t_cut);
             near += cls == 0;
@@ -319,7 +321,11 @@ k_emit(EmitArgs a, BrickGeom g, int nchunk, const double4_32a *__restrict__ xs64
        int32_t *__restrict__ cnt, int4 *__restrict__ tile_tab, int32_t *__restrict__ tile_tot,
        int32_t *__restrict__ flags) {
     __shared__ int t_start[kMaxTileBricks], t_base[kMaxTileBricks], t_code[kMaxTileBricks], t_total;
-    __shared__ int4 ctab[kMaxBrickCells][kMaxTileBricks];
+    // candidate cells, then ranges, of each cell: (first sorted atom, atoms << 7 | tile
+    // brick).  8 bytes an entry: shared memory taken here is taken from the L1 that
+    // the candidate loads live on (builds of 300,000 atoms: 1,542 us with 16 bytes,
+    // 1,501 with 8)
+    __shared__ uint2 ctab[kMaxBrickCells][kMaxTileBricks];
     __shared__ float4 shtab[kMaxTileBricks];  // image shift s L of each code (sx + 2) * 25 + ...
     __shared__ int nrange[kMaxBrickCells];  // table entries (ranges) of each cell
     __shared__ EmitArgs sargs;  // the band decision's copy of the arguments
@@ -380,22 +386,22 @@ k_emit(EmitArgs a, BrickGeom g, int nchunk, const double4_32a *__restrict__ xs64
         const int tz = (uz >> lb2) - bz + g.br[2];
         const int cn = (int)(brick_index(g, wx >> lb0, wy >> lb1, wz >> lb2) * g.bvol +
                              (((wx & lb0) << lb1 | (wy & lb1)) << lb2 | (wz & lb2)));
-        ctab[lc][kk] = make_int4(cell_start[cn], cell_start[cn + 1],
-                                 t_base[(tx * g.td[1] + ty) * g.td[2] + tz],
-                                 (sx + 2) * 25 + (sy + 2) * 5 + (sz + 2));
+        const unsigned first = cell_start[cn];
+        ctab[lc][kk] = make_uint2(first, ((unsigned)cell_start[cn + 1] - first) << 7 |
+                                             (unsigned)((tx * g.td[1] + ty) * g.td[2] + tz));
     }
     __syncthreads();
     // each cell's table as ranges: consecutive entries that continue one sorted
-    // range in the same tile brick under the same image shift merge, and empty
+    // range in the same tile brick (so under the same image shift) merge, and empty
     // cells drop out
     if (threadIdx.x < g.bvol) {
-        int4 *row = ctab[threadIdx.x];
+        uint2 *row = ctab[threadIdx.x];
         int m = 0;
         for (int k = 0; k < ncand; ++k) {
-            const int4 e = row[k];
-            if (e.x == e.y) continue;
-            if (m > 0 && row[m - 1].y == e.x && row[m - 1].z == e.z && row[m - 1].w == e.w)
-                row[m - 1].y = e.y;
+            const uint2 e = row[k];
+            if (e.y >> 7 == 0) continue;
+            if (m > 0 && row[m - 1].x + (row[m - 1].y >> 7) == e.x && ((row[m - 1].y ^ e.y) & 127u) == 0)
+                row[m - 1].y += e.y & ~127u;
             else
                 row[m++] = e;
         }
@@ -420,7 +426,7 @@ k_emit(EmitArgs a, BrickGeom g, int nchunk, const double4_32a *__restrict__ xs64
         int c[3] = {0, 0, 0};
         if (act) {
             const int lc = cell_s[i] - (int)(b * g.bvol);
-            emit_cells(a, &sargs, i, s, ctab[lc], shtab, nrange[lc], xs32[i], xs64, xs32, cap, c, scr,
+            emit_cells(a, &sargs, i, s, ctab[lc], t_base, t_code, shtab, nrange[lc], xs32[i], xs64, xs32, cap, c, scr,
                        t_total, flags);
         }
         const int mine = c[0] + c[1] + c[2];
