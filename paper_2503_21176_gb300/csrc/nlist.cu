@@ -199,7 +199,13 @@ constexpr int kCellDiv = 2;
 #ifndef QEQ_NL_UNROLL
 #define QEQ_NL_UNROLL 1
 #endif
-constexpr int kEmitThreads = 128;
+constexpr int kEmitThreads = 128;  // of the per-atom emit and the export
+// Block of the brick emit: ten warps of 8 rows, about a brick of water at r_list 9 A (73
+// rows), so that one round takes it; four warps took a third round nearly empty.
+// Builds of 60,000 / 120,000 / 300,000 atoms: 542 / 764 / 1,502 us with 4 warps, 500 /
+// 845 / 1,468 with 5, 415 / 734 / 1,512 with 8, 465 / 767 / 1,412 with 10, 437 / 756 /
+// 1,495 with 12, 451 / 772 / 1,866 with 16.
+constexpr int kBrickThreads = 320;
 constexpr int kEmitBlocksPerSm = 4;
 
 // s L for an image index s in [-2, 2]: exact in FP64 (a multiple of L by 0, 1 or
@@ -314,7 +320,7 @@ __device__ __forceinline__ void emit_cells(const EmitArgs &a, const EmitArgs *sa
 // take the brick's rows 8 at a time, kEmitLanes lanes a row.  The block also
 // records the largest tile and brick for the real-space launch, and writes no
 // entry when the tile exceeds 16-bit indices.
-__global__ void __launch_bounds__(kEmitThreads)
+__global__ void __launch_bounds__(kBrickThreads)
 k_emit(EmitArgs a, BrickGeom g, int nchunk, const double4_32a *__restrict__ xs64,
        const float4 *__restrict__ xs32, const int32_t *__restrict__ cell_s,
        const int32_t *__restrict__ cell_start, uint16_t *__restrict__ nbr, uint32_t *__restrict__ scr,
@@ -330,7 +336,7 @@ k_emit(EmitArgs a, BrickGeom g, int nchunk, const double4_32a *__restrict__ xs64
     __shared__ int nrange[kMaxBrickCells];  // table entries (ranges) of each cell
     __shared__ EmitArgs sargs;  // the band decision's copy of the arguments
     if (threadIdx.x == 0) sargs = a;
-    // nchunk blocks share a brick: chunk c takes the brick's groups of 32 rows
+    // nchunk blocks share a brick: chunk c takes the brick's groups of 80 rows
     // c, c + nchunk, ... (more blocks in flight for boxes of few bricks)
     const int64_t b = blockIdx.x / nchunk;
     const int chunk = (int)(blockIdx.x - b * nchunk);
@@ -1103,7 +1109,7 @@ static int launch_emit(qeq_ctx *ctx, cudaStream_t s) {
         return 1;
     }
     // blocks per brick: enough to put about kEmitBlocksPerSm blocks on every SM
-    // when the box has few bricks, at most one per 32 rows of the largest brick
+    // when the box has few bricks, at most one per 32 rows (four warps) of the largest brick
     // (from the previous build; 1.5 x the mean before the first)
     const int64_t nb = ctx->geom.nbricks;
     const int rows = ctx->max_rows > 0 ? ctx->max_rows
@@ -1111,7 +1117,7 @@ static int launch_emit(qeq_ctx *ctx, cudaStream_t s) {
     const int64_t want = (int64_t)kEmitBlocksPerSm * ctx->sm_count;
     const int nchunk = (int)std::max<int64_t>(
         1, std::min<int64_t>((want + nb - 1) / nb, (rows + 31) / 32));
-    k_emit<<<(unsigned)(nb * nchunk), kEmitThreads, 0, s>>>(
+    k_emit<<<(unsigned)(nb * nchunk), kBrickThreads, 0, s>>>(
         a, ctx->geom, nchunk, ctx->xs64, ctx->xs32, ctx->cell_s, ctx->cell_start, ctx->nbr,
         ctx->nbr_scratch, ctx->cnt, ctx->tile_tab, ctx->tile_tot, ctx->d_flags);
     return 1;
