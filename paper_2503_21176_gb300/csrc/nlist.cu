@@ -493,12 +493,12 @@ k_emit(EmitArgs a, BrickGeom g, int nchunk, const double4_32a *__restrict__ xs64
 // positions stay in registers), and its block.
 constexpr int kGroupRows = 4;
 constexpr int kGroupThreads = 256;
-// Systems below this many atoms per SM (38,912 on a 152-SM GB300) use it: there the
+// Systems below this many atoms per SM (10,944 on a 152-SM GB300) use it: there the
 // four-lane form leaves the chip idle and waits on its serial candidate loop.  Whole
-// builds, four lanes a row / grouped, r_list 9 A: 102 atoms 129 / 85 us, 648 153 / 92,
-// 3,000 202 / 117, 9,999 202 / 178, 20,001 319 / 319, 36,000 525 / 489, 60,000
-// 614 / 673, 300,000 1,622 / 2,548.
-constexpr int64_t kGroupAtomsPerSm = 256;
+// builds, four lanes a row / grouped, r_list 9 A: 102 atoms 129 / 82 us, 648 144 / 83,
+// 3,000 191 / 116, 9,999 184 / 177, 20,001 233 / 318, 36,000 354 / 487, 60,000
+// 465 / 669, 300,000 1,411 / 2,534.
+constexpr int64_t kGroupAtomsPerSm = 72;
 
 // Candidate ranges of one cell, built by one warp: its (2 reach + 1)^3 neighbour
 // cells in order, empty ones dropped and those that continue one sorted range in the

@@ -23,7 +23,7 @@ def _rows(s):
     ((400.0, 40.0, 9.0), 4.4, 0)])
 def test_large_lists_agree_with_the_atom_search(box, r_list, crowd):
     qg = cuda_or_skip()
-    n = 50_000  # above 256 atoms per SM
+    n = 50_000  # above the sizes of the grouped form
     rng = np.random.default_rng(n + crowd)
     box = np.array(box)
     R = rng.uniform(-0.2, 1.2, (n, 3)) * box
